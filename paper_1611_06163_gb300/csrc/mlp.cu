@@ -29,237 +29,358 @@ constexpr int TPB = 128;
 
 __device__ __forceinline__ float bf16r(float x) { return __bfloat162float(__float2bfloat16_rn(x)); }
 
-__device__ __forceinline__ float gelu(float z) { return 0.5f * z * (1.0f + erff(z * 0.70710678118654752f)); }
+// The shared part of both kernels. A CTA of TPB threads works on CH samples of
+// one member as small matrix products from shared memory: thread t owns the
+// samples s0..s0+3 (s0 = 4 (t & 7)) and, of the 64 features, 4 to..4 to + 3
+// (to = t >> 3) in the products that end in layer 1 and to, to + 16, ... in
+// those that end in layer 2 (the strided rows keep the 68-float weight rows on
+// distinct banks). A 4 x 4 tile per thread takes 8 16-byte shared loads per 64
+// multiply-adds.
+constexpr int CH = 32;           // samples per CTA
+constexpr int LDS_ = CH + 4;     // padded row of a feature-major activation (16-byte rows)
+constexpr int LDW = HID + 4;     // padded row of W2
 
-__device__ __forceinline__ float gelu_grad(float z)
+struct NetSmem {
+    float W2[HID][LDW];
+    float W1[HID][IN];
+    float b1[HID], b2[HID], W3[OUT][HID], b3[OUT], pad[2];
+    float X[IN][LDS_];
+    float H1[HID][LDS_];
+    float Y[TPB / 32][OUT][CH];  // each warp's share of the outputs
+};
+
+__device__ __forceinline__ void load_net(NetSmem &S, const float *__restrict__ p)
 {
-    return 0.5f * (1.0f + erff(z * 0.70710678118654752f)) + z * expf(-0.5f * z * z) * 0.39894228040143268f;
+    const int t = threadIdx.x;
+    for (int k = t; k < HID * HID; k += TPB) S.W2[k >> 6][k & 63] = bf16r(p[OW2 + k]);
+    for (int k = t; k < HID * IN; k += TPB) S.W1[k >> 2][k & 3] = bf16r(p[OW1 + k]);
+    if (t < HID) {
+        S.b1[t] = bf16r(p[OB1 + t]);
+        S.b2[t] = bf16r(p[OB2 + t]);
+        S.W3[0][t] = bf16r(p[OW3 + t]);
+        S.W3[1][t] = bf16r(p[OW3 + HID + t]);
+        if (t < OUT) S.b3[t] = bf16r(p[OB3 + t]);
+    }
 }
 
-__device__ void load_weights(float *w, const float *params)
+__device__ __forceinline__ float4 ld4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
+__device__ __forceinline__ void st4(float *p, float a, float b, float c, float d)
 {
-    for (int k = threadIdx.x; k < NP; k += blockDim.x) w[k] = bf16r(params[k]);
+    *reinterpret_cast<float4 *>(p) = make_float4(a, b, c, d);
+}
+
+// GELU of z and (GRAD) its derivative, one error function for both.
+template <bool GRAD>
+__device__ __forceinline__ float gelu_both(float z, float &g)
+{
+    const float e = 1.0f + erff(z * 0.70710678118654752f);
+    if (GRAD) g = 0.5f * e + z * expf(-0.5f * z * z) * 0.39894228040143268f;
+    return 0.5f * z * e;
+}
+
+// Forward pass: h2[q][r] of feature to + 16 q and sample s0 + r, the
+// derivatives g1[u][r] (feature 4 to + u) and g2[q][r], H1 and the warps' shares
+// of the outputs in shared memory (complete after the caller's barrier).
+template <bool GRAD>
+__device__ __forceinline__ void forward(NetSmem &S, int s0, int to, float (&g1)[4][4], float (&h2)[4][4],
+                                        float (&g2)[4][4])
+{
+    {
+        float4 x[IN];
+#pragma unroll
+        for (int c = 0; c < IN; ++c) x[c] = ld4(&S.X[c][s0]);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int o = 4 * to + u;
+            const float4 w = ld4(S.W1[o]);
+            const float b = S.b1[o];
+            float z[4] = {b, b, b, b}, h[4];
+            const float wc[IN] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+            for (int c = 0; c < IN; ++c) {
+                z[0] = fmaf(wc[c], x[c].x, z[0]);
+                z[1] = fmaf(wc[c], x[c].y, z[1]);
+                z[2] = fmaf(wc[c], x[c].z, z[2]);
+                z[3] = fmaf(wc[c], x[c].w, z[3]);
+            }
+#pragma unroll
+            for (int r = 0; r < 4; ++r) h[r] = gelu_both<GRAD>(z[r], g1[u][r]);
+            st4(&S.H1[o][s0], h[0], h[1], h[2], h[3]);
+        }
+    }
     __syncthreads();
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const float b = S.b2[to + 16 * q];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) h2[q][r] = b;
+    }
+#pragma unroll 4
+    for (int i = 0; i < HID; i += 4) {
+        float4 w[4], h[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) w[q] = ld4(&S.W2[to + 16 * q][i]);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) h[u] = ld4(&S.H1[i + u][s0]);
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const float wv = u == 0 ? w[q].x : u == 1 ? w[q].y : u == 2 ? w[q].z : w[q].w;
+                h2[q][0] = fmaf(wv, h[u].x, h2[q][0]);
+                h2[q][1] = fmaf(wv, h[u].y, h2[q][1]);
+                h2[q][2] = fmaf(wv, h[u].z, h2[q][2]);
+                h2[q][3] = fmaf(wv, h[u].w, h2[q][3]);
+            }
+    }
+    float y[OUT][4];
+#pragma unroll
+    for (int k = 0; k < OUT; ++k)
+#pragma unroll
+        for (int r = 0; r < 4; ++r) y[k][r] = 0.0f;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const float w0 = S.W3[0][to + 16 * q], w1 = S.W3[1][to + 16 * q];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            h2[q][r] = gelu_both<GRAD>(h2[q][r], g2[q][r]);
+            y[0][r] = fmaf(w0, h2[q][r], y[0][r]);
+            y[1][r] = fmaf(w1, h2[q][r], y[1][r]);
+        }
+    }
+    // the four features' groups of the warp (lane bits 3 and 4)
+#pragma unroll
+    for (int k = 0; k < OUT; ++k)
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            y[k][r] += __shfl_xor_sync(0xffffffffu, y[k][r], 8);
+            y[k][r] += __shfl_xor_sync(0xffffffffu, y[k][r], 16);
+        }
+    if ((threadIdx.x & 24) == 0)
+#pragma unroll
+        for (int k = 0; k < OUT; ++k) st4(&S.Y[threadIdx.x >> 5][k][s0], y[k][0], y[k][1], y[k][2], y[k][3]);
 }
 
-// Forward pass (prediction) of one sample per thread.
+// Output k of sample s: the bias and the warps' shares in warp order.
+__device__ __forceinline__ float output(const NetSmem &S, int k, int s)
+{
+    float y = S.b3[k];
+#pragma unroll
+    for (int w = 0; w < TPB / 32; ++w) y += S.Y[w][k][s];
+    return y;
+}
+
+// Prediction: the CTA's CH samples through one member. Bound by the two
+// products' multiply-adds and the error function; 2048 samples x 5 members: 320
+// CTAs, all resident.
 __global__ void __launch_bounds__(TPB) k_mlp_fwd(const float *__restrict__ params, const float *__restrict__ X,
                                                  int n, float *Y)
 {
-    __shared__ float w[NP];
-    const int mbr = blockIdx.y;
-    load_weights(w, params + (size_t)mbr * NP);
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= n) return;
-    float x[IN];
-#pragma unroll
-    for (int i = 0; i < IN; ++i) x[i] = X[(size_t)s * IN + i];
-    float h1[HID];
-#pragma unroll
-    for (int o = 0; o < HID; ++o) {
-        float z = w[OB1 + o];
-#pragma unroll
-        for (int i = 0; i < IN; ++i) z = fmaf(w[OW1 + o * IN + i], x[i], z);
-        h1[o] = gelu(z);
+    __shared__ NetSmem S;
+    const int mbr = blockIdx.y, t = threadIdx.x;
+    load_net(S, params + (size_t)mbr * NP);
+    {
+        const int s = t >> 2, c = t & 3, smp = blockIdx.x * CH + s;
+        S.X[c][s] = smp < n ? X[(size_t)smp * IN + c] : 0.0f;
     }
-    float y0 = w[OB3], y1 = w[OB3 + 1];
-    // four outputs at a time: four independent multiply-add chains
-    for (int o0 = 0; o0 < HID; o0 += 4) {
-        float z[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) z[q] = w[OB2 + o0 + q];
-#pragma unroll
-        for (int i = 0; i < HID; ++i)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) z[q] = fmaf(w[OW2 + (o0 + q) * HID + i], h1[i], z[q]);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const float h = gelu(z[q]);
-            y0 = fmaf(w[OW3 + o0 + q], h, y0);
-            y1 = fmaf(w[OW3 + HID + o0 + q], h, y1);
-        }
-    }
-    const size_t yo = ((size_t)mbr * n + s) * OUT;
-    Y[yo] = y0;
-    Y[yo + 1] = y1;
+    __syncthreads();
+    float g1[4][4], g2[4][4], h2[4][4];
+    forward<false>(S, 4 * (t & 7), t >> 3, g1, h2, g2);
+    __syncthreads();
+    const int s = t >> 1, k = t & 1, smp = blockIdx.x * CH + s;
+    if (s < CH && smp < n) Y[((size_t)mbr * n + smp) * OUT + k] = output(S, k, s);
 }
 
-// One training pass over a chunk of CH samples (one per thread) of one
-// member: forward, back-propagation, and the chunk's share of every
-// parameter's gradient, in one launch. The chunk's activations and error
-// signals stay in shared memory, feature-major with rows padded to CH + 1 so
-// that the per-sample writes and the per-parameter reads are free of bank
-// conflicts. Each gradient entry is the chunk's samples summed in sample
-// order; k_mlp_reduce adds the chunks in chunk order (float-float), so the
-// gradient is deterministic.
-constexpr int CH = 128;
-constexpr int LD = CH + 1;
-
-struct ChunkSmem {
-    float w[NP];
-    float X[IN][LD];
-    float H1[HID][LD], A1[HID][LD];   // A1: z1, then the error signal d1
-    float H2[HID][LD], A2[HID][LD];   // A2: z2, then the error signal d2
-    float D3[OUT][LD];
-    float red[CH / 32];
+// One training pass over a chunk of CH samples of one member: forward,
+// back-propagation, and the chunk's share of every parameter's gradient, in one
+// launch. The error signals of layer 2 and the activations of layer 1 meet in
+// shared memory for the 64 x 64 gradient; everything else stays in registers
+// and is summed over the chunk's samples by shuffles in a fixed tree.
+// k_mlp_reduce adds the chunks in a fixed order (float-float), so the gradient
+// is deterministic.
+// Bound by the multiply-adds (3 x 4096 per sample) and the error functions
+// (128 per sample); about 5300 instructions per warp. Chunks of 32 samples at
+// 128 threads put four or five CTAs of 40 KB on each SM for 5 x 4096 samples: 25
+// us (one thread per sample with 154 KB of shared memory left four warps on an SM
+// and a second, nearly empty wave: 88 us); 49 % of the issue slots.
+struct TrainSmem {
+    NetSmem N;
+    float D2[HID][LDS_];
 };
 
-__global__ void __launch_bounds__(CH) k_mlp_chunk(const float *__restrict__ params, const float *__restrict__ X,
-                                                 const float *__restrict__ T, int n, float *part, float *loss_part)
+__global__ void __launch_bounds__(TPB, 5) k_mlp_chunk(const float *__restrict__ params, const float *__restrict__ X,
+                                                      const float *__restrict__ T, int n, float *part,
+                                                      float *loss_part)
 {
-    extern __shared__ float4 smem_raw[];
-    ChunkSmem &S = *reinterpret_cast<ChunkSmem *>(smem_raw);
+    __shared__ TrainSmem Q;
+    NetSmem &S = Q.N;
     const int mbr = blockIdx.y, c = blockIdx.x, nch = gridDim.x;
     const int t = threadIdx.x;
-    const int smp = c * CH + t;
-    const bool valid = smp < n;
-    for (int k = t; k < NP; k += CH) S.w[k] = bf16r(params[(size_t)mbr * NP + k]);
+    const int s0 = 4 * (t & 7), to = t >> 3;
+    {
+        // the samples do not depend on the previous launch, the weights do
+        const int s = t >> 2, k = t & 3, smp = c * CH + s;
+        S.X[k][s] = smp < n ? X[(size_t)smp * IN + k] : 0.0f;
+    }
+    pdl_enter();
+    load_net(S, params + (size_t)mbr * NP);
     __syncthreads();
-    const float *w = S.w;
+    float g1[4][4], g2[4][4], h2[4][4];
+    forward<true>(S, s0, to, g1, h2, g2);
+    __syncthreads();
 
-    // ---- forward
-    float x[IN];
+    float d3[OUT][4], err2 = 0.0f;
+    const float sc = 2.0f / (float)(n * OUT);
 #pragma unroll
-    for (int i = 0; i < IN; ++i) {
-        x[i] = valid ? X[(size_t)smp * IN + i] : 0.0f;
-        S.X[i][t] = x[i];
+    for (int r = 0; r < 4; ++r) {
+        const int smp = c * CH + s0 + r;
+        const bool valid = smp < n;
+        const float2 y = valid ? *reinterpret_cast<const float2 *>(T + (size_t)smp * OUT) : make_float2(0.f, 0.f);
+        const float e0 = output(S, 0, s0 + r) - y.x, e1 = output(S, 1, s0 + r) - y.y;
+        d3[0][r] = valid ? sc * e0 : 0.0f;
+        d3[1][r] = valid ? sc * e1 : 0.0f;
+        err2 += valid ? e0 * e0 + e1 * e1 : 0.0f;
     }
-    float h1[HID];
-#pragma unroll
-    for (int o = 0; o < HID; ++o) {
-        float z = w[OB1 + o];
-#pragma unroll
-        for (int i = 0; i < IN; ++i) z = fmaf(w[OW1 + o * IN + i], x[i], z);
-        h1[o] = valid ? gelu(z) : 0.0f;
-        S.A1[o][t] = z;
-        S.H1[o][t] = h1[o];
-    }
-    float y0 = w[OB3], y1 = w[OB3 + 1];
-    for (int o0 = 0; o0 < HID; o0 += 4) {
-        float z[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) z[q] = w[OB2 + o0 + q];
-#pragma unroll
-        for (int i = 0; i < HID; ++i)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) z[q] = fmaf(w[OW2 + (o0 + q) * HID + i], h1[i], z[q]);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int o = o0 + q;
-            const float h = valid ? gelu(z[q]) : 0.0f;
-            S.A2[o][t] = z[q];
-            S.H2[o][t] = h;
-            y0 = fmaf(w[OW3 + o], h, y0);
-            y1 = fmaf(w[OW3 + HID + o], h, y1);
+    float *out = part + ((size_t)mbr * nch + c) * NP;
+    // sum of a value over the chunk's samples: the thread's four, then the
+    // eight sample groups of the feature (lane bits 0-2)
+    auto over_samples = [](float v) {
+        v += __shfl_xor_sync(0xffffffffu, v, 1);
+        v += __shfl_xor_sync(0xffffffffu, v, 2);
+        v += __shfl_xor_sync(0xffffffffu, v, 4);
+        return v;
+    };
+    const bool writer = (t & 7) == 0;
+    {
+        const float l = over_samples(err2), b0 = over_samples((d3[0][0] + d3[0][1]) + (d3[0][2] + d3[0][3])),
+                    b1 = over_samples((d3[1][0] + d3[1][1]) + (d3[1][2] + d3[1][3]));
+        if (t == 0) {
+            loss_part[(size_t)mbr * nch + c] = l;
+            out[OB3] = b0;
+            out[OB3 + 1] = b1;
         }
     }
-    float d30 = 0.0f, d31 = 0.0f, err2 = 0.0f;
-    if (valid) {
-        const float e0 = y0 - T[(size_t)smp * OUT], e1 = y1 - T[(size_t)smp * OUT + 1];
-        const float sc = 2.0f / (float)(n * OUT);
-        d30 = sc * e0;
-        d31 = sc * e1;
-        err2 = e0 * e0 + e1 * e1;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int o = to + 16 * q;
+        const float w0 = S.W3[0][o], w1 = S.W3[1][o];
+        float d2[4], a0 = 0.0f, a1 = 0.0f;
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            d2[r] = fmaf(d3[0][r], w0, d3[1][r] * w1) * g2[q][r];
+            a0 = fmaf(d3[0][r], h2[q][r], a0);
+            a1 = fmaf(d3[1][r], h2[q][r], a1);
+        }
+        st4(&Q.D2[o][s0], d2[0], d2[1], d2[2], d2[3]);
+        a0 = over_samples(a0);
+        a1 = over_samples(a1);
+        const float b2 = over_samples((d2[0] + d2[1]) + (d2[2] + d2[3]));
+        if (writer) {
+            out[OW3 + o] = a0;
+            out[OW3 + HID + o] = a1;
+            out[OB2 + o] = b2;
+        }
     }
-    S.D3[0][t] = d30;
-    S.D3[1][t] = d31;
-
-    // ---- back-propagation (this thread's sample)
-    float d2[HID];
-#pragma unroll
-    for (int o = 0; o < HID; ++o) {
-        const float g = fmaf(d30, w[OW3 + o], d31 * w[OW3 + HID + o]);
-        d2[o] = g * gelu_grad(S.A2[o][t]);
-        S.A2[o][t] = d2[o];
-    }
-    for (int i0 = 0; i0 < HID; i0 += 4) {
-        float a[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-#pragma unroll
-        for (int o = 0; o < HID; ++o)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) a[q] = fmaf(d2[o], w[OW2 + o * HID + i0 + q], a[q]);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) S.A1[i0 + q][t] = a[q] * gelu_grad(S.A1[i0 + q][t]);
-    }
-    for (int o = 16; o > 0; o >>= 1) err2 += __shfl_down_sync(0xffffffffu, err2, o);
-    if ((t & 31) == 0) S.red[t >> 5] = err2;
     __syncthreads();
-
-    // ---- the chunk's gradient: sums over its samples in sample order
-    float *out = part + ((size_t)mbr * nch + c) * NP;
     {
-        // dW2[o][i] = sum_s d2[o][s] h1[i][s]: a 4 x 8 tile per thread
-        const int o0 = 4 * (t >> 3), i0 = 8 * (t & 7);
+        // error signals of layer 1: features 4 to + u
+        float a[4][4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+            for (int r = 0; r < 4; ++r) a[u][r] = 0.0f;
+#pragma unroll 8
+        for (int o = 0; o < HID; ++o) {
+            const float4 w = ld4(&S.W2[o][4 * to]), d = ld4(&Q.D2[o][s0]);
+            const float wv[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                a[u][0] = fmaf(d.x, wv[u], a[u][0]);
+                a[u][1] = fmaf(d.y, wv[u], a[u][1]);
+                a[u][2] = fmaf(d.z, wv[u], a[u][2]);
+                a[u][3] = fmaf(d.w, wv[u], a[u][3]);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int i = 4 * to + u;
+            float d1[4], b = 0.0f;
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                d1[r] = a[u][r] * g1[u][r];
+                b += d1[r];
+            }
+            b = over_samples(b);
+            float w1[IN];
+#pragma unroll
+            for (int k = 0; k < IN; ++k) {
+                const float4 x = ld4(&S.X[k][s0]);
+                w1[k] = over_samples(fmaf(d1[3], x.w, fmaf(d1[2], x.z, fmaf(d1[1], x.y, d1[0] * x.x))));
+            }
+            if (writer) {
+                out[OB1 + i] = b;
+#pragma unroll
+                for (int k = 0; k < IN; ++k) out[OW1 + i * IN + k] = w1[k];
+            }
+        }
+    }
+    {
+        // dW2[o][i] = sum_s d2[o][s] h1[i][s]: features o = to + 16 q of layer
+        // 2 and i = (t & 7) + 8 p of layer 1
+        const int ii = t & 7;
         float acc[4][8];
 #pragma unroll
-        for (int a = 0; a < 4; ++a)
+        for (int q = 0; q < 4; ++q)
 #pragma unroll
-            for (int b = 0; b < 8; ++b) acc[a][b] = 0.0f;
-        for (int k = 0; k < CH; ++k) {
-            float da[4], hb[8];
+            for (int p = 0; p < 8; ++p) acc[q][p] = 0.0f;
+#pragma unroll 2
+        for (int s = 0; s < CH; s += 4) {
+            float4 d[4];
 #pragma unroll
-            for (int a = 0; a < 4; ++a) da[a] = S.A2[o0 + a][k];
+            for (int q = 0; q < 4; ++q) d[q] = ld4(&Q.D2[to + 16 * q][s]);
 #pragma unroll
-            for (int b = 0; b < 8; ++b) hb[b] = S.H1[i0 + b][k];
+            for (int p = 0; p < 8; ++p) {
+                const float4 h = ld4(&S.H1[ii + 8 * p][s]);
 #pragma unroll
-            for (int a = 0; a < 4; ++a)
-#pragma unroll
-                for (int b = 0; b < 8; ++b) acc[a][b] = fmaf(da[a], hb[b], acc[a][b]);
+                for (int q = 0; q < 4; ++q)
+                    acc[q][p] = fmaf(d[q].w, h.w, fmaf(d[q].z, h.z, fmaf(d[q].y, h.y, fmaf(d[q].x, h.x, acc[q][p]))));
+            }
         }
 #pragma unroll
-        for (int a = 0; a < 4; ++a)
+        for (int q = 0; q < 4; ++q)
 #pragma unroll
-            for (int b = 0; b < 8; ++b) out[OW2 + (o0 + a) * HID + i0 + b] = acc[a][b];
-    }
-    if (t < HID) {
-        // row o of dW1, db1 and db2
-        const int o = t;
-        float g1[IN] = {0.0f, 0.0f, 0.0f, 0.0f}, gb1 = 0.0f, gb2 = 0.0f;
-        for (int k = 0; k < CH; ++k) {
-            const float d1 = S.A1[o][k];
-#pragma unroll
-            for (int i = 0; i < IN; ++i) g1[i] = fmaf(d1, S.X[i][k], g1[i]);
-            gb1 += d1;
-            gb2 += S.A2[o][k];
-        }
-#pragma unroll
-        for (int i = 0; i < IN; ++i) out[OW1 + o * IN + i] = g1[i];
-        out[OB1 + o] = gb1;
-        out[OB2 + o] = gb2;
-    } else {
-        // column i of dW3, and db3
-        const int i = t - HID;
-        float g0 = 0.0f, g1 = 0.0f, gb = 0.0f;
-        for (int k = 0; k < CH; ++k) {
-            const float h = S.H2[i][k];
-            g0 = fmaf(S.D3[0][k], h, g0);
-            g1 = fmaf(S.D3[1][k], h, g1);
-            if (i < OUT) gb += S.D3[i][k];
-        }
-        out[OW3 + i] = g0;
-        out[OW3 + HID + i] = g1;
-        if (i < OUT) out[OB3 + i] = gb;
-    }
-    if (t == 0) {
-        float l = 0.0f;
-        for (int k = 0; k < CH / 32; ++k) l += S.red[k];
-        loss_part[(size_t)mbr * nch + c] = l;
+            for (int p = 0; p < 8; ++p) out[OW2 + (to + 16 * q) * HID + ii + 8 * p] = acc[q][p];
     }
 }
 
-// Each parameter's gradient: its chunks' sums added in chunk order
-// (float-float); with adam, the Adam step (Kingma & Ba) on the float master
-// weights, bc1 and bc2 being the bias corrections 1 - beta^t.
-__global__ void __launch_bounds__(TPB) k_mlp_reduce(const float *__restrict__ part, int nch, int total,
-                                                    float *grad, int adam, float *params, float *m, float *v,
-                                                    float lr, float beta1, float beta2, float eps, float bc1,
-                                                    float bc2)
+// Each parameter's gradient: its chunks' sums added in float-float, eight warps
+// taking every eighth chunk and their sums added in warp order (a fixed order
+// for a given chunk count; 32 parameters per CTA, so a warp reads 128 bytes per
+// chunk and the eight warps keep enough loads in flight: 12 MB for 5 x 4096
+// samples, 6.5 us). With adam, the Adam step (Kingma & Ba) on the float master weights,
+// bc1 and bc2 being the bias corrections 1 - beta^t.
+constexpr int RED_WARPS = 8;
+__global__ void __launch_bounds__(32 * RED_WARPS) k_mlp_reduce(const float *__restrict__ part, int nch, int total,
+                                                               float *grad, int adam, float *params, float *m,
+                                                               float *v, float lr, float beta1, float beta2,
+                                                               float eps, float bc1, float bc2)
 {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= total) return;
-    const int mbr = k / NP, p = k - mbr * NP;
+    pdl_enter();
+    __shared__ FF sum[RED_WARPS][32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int k = blockIdx.x * 32 + lane;
     FF acc{0.0f, 0.0f};
-    for (int c = 0; c < nch; ++c) acc = ff_add(acc, part[((size_t)mbr * nch + c) * NP + p]);
+    if (k < total) {
+        const int mbr = k / NP;
+        const float *p = part + (size_t)mbr * nch * NP + (k - mbr * NP);
+#pragma unroll 8
+        for (int c = w; c < nch; c += RED_WARPS) acc = ff_add(acc, p[(size_t)c * NP]);
+    }
+    sum[w][lane] = acc;
+    __syncthreads();
+    if (w != 0 || k >= total) return;
+#pragma unroll
+    for (int u = 1; u < RED_WARPS; ++u) acc = ff_add(acc, sum[u][lane]);
     const float g = acc.hi + acc.lo;
     grad[k] = g;
     if (adam) {
@@ -331,14 +452,8 @@ tdpd_status alloc_data(tdpd_mlp *m, int n)
 // lr > 0, one Adam step); loss (may be NULL) receives each member's loss.
 tdpd_status pass(tdpd_mlp *m, float lr, double *loss)
 {
-    static bool attr = false;
-    if (!attr) {
-        MCU(cudaFuncSetAttribute(k_mlp_chunk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(ChunkSmem)));
-        attr = true;
-    }
     const int nch = (m->n + CH - 1) / CH;
-    k_mlp_chunk<<<dim3(nch, m->members), CH, sizeof(ChunkSmem), m->st>>>(m->params, m->X, m->T, m->n, m->gpart,
-                                                                          m->loss_part);
+    launch_pdl(k_mlp_chunk, dim3(nch, m->members), TPB, m->st, m->params, m->X, m->T, m->n, m->gpart, m->loss_part);
     const int total = m->members * NP;
     float bc1 = 1.0f, bc2 = 1.0f;
     if (lr > 0.0f) {
@@ -346,9 +461,8 @@ tdpd_status pass(tdpd_mlp *m, float lr, double *loss)
         bc1 = (float)(1.0 - std::pow(0.9, (double)m->t));
         bc2 = (float)(1.0 - std::pow(0.999, (double)m->t));
     }
-    k_mlp_reduce<<<(total + TPB - 1) / TPB, TPB, 0, m->st>>>(m->gpart, nch, total, m->grad, lr > 0.0f ? 1 : 0,
-                                                             m->params, m->m, m->v, lr, 0.9f, 0.999f, 1e-8f, bc1,
-                                                             bc2);
+    launch_pdl(k_mlp_reduce, (total + 31) / 32, 32 * RED_WARPS, m->st, m->gpart, nch, total, m->grad,
+               lr > 0.0f ? 1 : 0, m->params, m->m, m->v, lr, 0.9f, 0.999f, 1e-8f, bc1, bc2);
     MCU(cudaGetLastError());
     if (loss) {
         std::vector<float> part((size_t)m->members * nch);
@@ -487,7 +601,7 @@ tdpd_status tdpd_mlp_predict(tdpd_mlp *m, int n, const float *X, float *mean, fl
     for (int i = 0; i < n; ++i)
         for (int c = 0; c < IN; ++c) xs[(size_t)i * IN + c] = (float)((X[(size_t)i * IN + c] - m->mx[c]) / m->sx[c]);
     MCU(cudaMemcpyAsync(dX, xs.data(), xs.size() * sizeof(float), cudaMemcpyHostToDevice, m->st));
-    k_mlp_fwd<<<dim3((n + TPB - 1) / TPB, m->members), TPB, 0, m->st>>>(m->params, dX, n, dY);
+    k_mlp_fwd<<<dim3((n + CH - 1) / CH, m->members), TPB, 0, m->st>>>(m->params, dX, n, dY);
     MCU(cudaGetLastError());
     MCU(cudaMemcpyAsync(ys.data(), dY, ys.size() * sizeof(float), cudaMemcpyDeviceToHost, m->st));
     MCU(cudaFreeAsync(dX, m->st));
