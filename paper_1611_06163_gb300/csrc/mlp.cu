@@ -29,6 +29,11 @@ constexpr int TPB = 128;
 
 __device__ __forceinline__ float bf16r(float x) { return __bfloat162float(__float2bfloat16_rn(x)); }
 
+// Means and deviations of the training set's inputs and outputs.
+struct Standard {
+    double mx[IN], sx[IN], my[OUT], sy[OUT];
+};
+
 // The shared part of both kernels. A CTA of TPB threads works on CH samples of
 // one member as small matrix products from shared memory: thread t owns the
 // samples s0..s0+3 (s0 = 4 (t & 7)) and, of the 64 features, 4 to..4 to + 3
@@ -170,18 +175,19 @@ __device__ __forceinline__ float output(const NetSmem &S, int k, int s)
     return y;
 }
 
-// Prediction: the CTA's CH samples through one member. Bound by the two
-// products' multiply-adds and the error function; 2048 samples x 5 members: 320
-// CTAs, all resident.
+// Prediction: the CTA's CH samples through one member; X: raw inputs,
+// standardised here in binary64 and rounded once. Bound by the two products'
+// multiply-adds and the error function; 2048 samples x 5 members: 320 CTAs, all
+// resident.
 __global__ void __launch_bounds__(TPB) k_mlp_fwd(const float *__restrict__ params, const float *__restrict__ X,
-                                                 int n, float *Y)
+                                                 Standard st, int n, float *Y)
 {
     __shared__ NetSmem S;
     const int mbr = blockIdx.y, t = threadIdx.x;
     load_net(S, params + (size_t)mbr * NP);
     {
         const int s = t >> 2, c = t & 3, smp = blockIdx.x * CH + s;
-        S.X[c][s] = smp < n ? X[(size_t)smp * IN + c] : 0.0f;
+        S.X[c][s] = smp < n ? (float)((X[(size_t)smp * IN + c] - st.mx[c]) / st.sx[c]) : 0.0f;
     }
     __syncthreads();
     float g1[4][4], g2[4][4], h2[4][4];
@@ -189,6 +195,28 @@ __global__ void __launch_bounds__(TPB) k_mlp_fwd(const float *__restrict__ param
     __syncthreads();
     const int s = t >> 1, k = t & 1, smp = blockIdx.x * CH + s;
     if (s < CH && smp < n) Y[((size_t)mbr * n + smp) * OUT + k] = output(S, k, s);
+}
+
+// Ensemble statistics of the predictions in binary64: Y becomes each member's
+// output in raw units, mean and rel the ensemble's mean and relative spread.
+__global__ void __launch_bounds__(TPB) k_mlp_stats(float *Y, Standard st, int members, int n, float *mean, float *rel)
+{
+    pdl_enter();
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;      // (sample, output)
+    if (e >= n * OUT) return;
+    const int c = e % OUT;
+    double s = 0.0, s2 = 0.0;
+    for (int k = 0; k < members; ++k) {
+        const size_t at = (size_t)k * n * OUT + e;
+        const double y = Y[at] * st.sy[c] + st.my[c];
+        Y[at] = (float)y;
+        s += y;
+        s2 += y * y;
+    }
+    const double mu = s / members;
+    const double var = members > 1 ? fmax(0.0, (s2 - members * mu * mu) / (members - 1)) : 0.0;
+    mean[e] = (float)mu;
+    rel[e] = (float)(sqrt(var) / fmax(fabs(mu), 1e-30));
 }
 
 // One training pass over a chunk of CH samples of one member: forward,
@@ -400,7 +428,12 @@ struct tdpd_mlp {
     float *params = nullptr, *m = nullptr, *v = nullptr, *grad = nullptr;
     float *X = nullptr, *T = nullptr, *loss_part = nullptr;
     float *gpart = nullptr;     // [members][chunks][NP] per-chunk gradient sums
-    double mx[IN] = {}, sx[IN] = {}, my[OUT] = {}, sy[OUT] = {};
+    Standard sd = {};
+    float *base = nullptr;      // one allocation: params, m, v, grad, the first workspace
+    // prediction workspace, kept between calls up to PRED_KEEP floats: inputs,
+    // then mean, relative spread and the members' outputs
+    float *pred = nullptr, *pred_own = nullptr;
+    size_t pred_floats = 0;
     bool have_data = false;
     cudaStream_t st = nullptr;
     std::vector<void *> data_allocs;
@@ -448,6 +481,25 @@ tdpd_status alloc_data(tdpd_mlp *m, int n)
     return TDPD_OK;
 }
 
+// The prediction workspace, at least `need` floats: PRED_MIN of them come with
+// the handle, more are allocated once. (Two allocations and their release on every
+// call, the standardisation and the ensemble statistics on the host took 250 us of
+// a call that ranks 2048 points with five members.)
+constexpr size_t PRED_MIN = (size_t)1 << 17, PRED_KEEP = (size_t)1 << 22;
+tdpd_status pred_workspace(tdpd_mlp *m, size_t need)
+{
+    if (need <= m->pred_floats) return TDPD_OK;
+    void *d = nullptr;
+    if (cudaMalloc(&d, need * sizeof(float)) != cudaSuccess) {
+        cudaGetLastError();
+        return mfail(TDPD_ENOMEM, "tdpd_mlp_predict: device allocation failed");
+    }
+    if (m->pred_own) cudaFree(m->pred_own);       // (every call waits for its work)
+    m->pred = m->pred_own = (float *)d;
+    m->pred_floats = need;
+    return TDPD_OK;
+}
+
 // One pass over the data: the chunks' gradients, then their sums (and, with
 // lr > 0, one Adam step); loss (may be NULL) receives each member's loss.
 tdpd_status pass(tdpd_mlp *m, float lr, double *loss)
@@ -488,22 +540,21 @@ tdpd_status tdpd_mlp_create(tdpd_mlp **out, int members)
     tdpd_mlp *m = new (std::nothrow) tdpd_mlp;
     if (!m) return mfail(TDPD_ENOMEM, "host allocation failed");
     m->members = members;
-    const size_t bytes = (size_t)members * NP * sizeof(float);
-    void *p[4] = {};
-    for (int k = 0; k < 4; ++k)
-        if (cudaMalloc(&p[k], bytes) != cudaSuccess) {
-            for (int j = 0; j < k; ++j) cudaFree(p[j]);
-            delete m;
-            return mfail(TDPD_ENOMEM, "tdpd_mlp_create: device allocation failed");
-        }
-    m->params = (float *)p[0];
-    m->m = (float *)p[1];
-    m->v = (float *)p[2];
-    m->grad = (float *)p[3];
+    const size_t par = (size_t)members * NP;
+    void *p = nullptr;
+    if (cudaMalloc(&p, (4 * par + PRED_MIN) * sizeof(float)) != cudaSuccess) {
+        delete m;
+        return mfail(TDPD_ENOMEM, "tdpd_mlp_create: device allocation failed");
+    }
+    m->base = m->params = (float *)p;
+    m->m = m->params + par;
+    m->v = m->m + par;
+    m->grad = m->v + par;
+    m->pred = m->grad + par;
+    m->pred_floats = PRED_MIN;
     if (cudaStreamCreateWithFlags(&m->st, cudaStreamNonBlocking) != cudaSuccess ||
-        cudaMemset(m->params, 0, bytes) != cudaSuccess || cudaMemset(m->m, 0, bytes) != cudaSuccess ||
-        cudaMemset(m->v, 0, bytes) != cudaSuccess) {
-        for (int k = 0; k < 4; ++k) cudaFree(p[k]);
+        cudaMemset(m->params, 0, 3 * par * sizeof(float)) != cudaSuccess) {
+        cudaFree(m->base);
         delete m;
         return mfail(TDPD_ECUDA, "tdpd_mlp_create: stream or memset failed");
     }
@@ -548,13 +599,13 @@ tdpd_status tdpd_mlp_set_data(tdpd_mlp *m, int n, const float *X, const float *Y
             s2 += d * d;
         }
         const double sd = std::sqrt(s2 / n) + 1e-12;
-        if (k < IN) { m->mx[c] = mean; m->sx[c] = sd; }
-        else { m->my[c] = mean; m->sy[c] = sd; }
+        if (k < IN) { m->sd.mx[c] = mean; m->sd.sx[c] = sd; }
+        else { m->sd.my[c] = mean; m->sd.sy[c] = sd; }
     }
     std::vector<float> xs((size_t)n * IN), ys((size_t)n * OUT);
     for (int i = 0; i < n; ++i) {
-        for (int c = 0; c < IN; ++c) xs[(size_t)i * IN + c] = (float)((X[(size_t)i * IN + c] - m->mx[c]) / m->sx[c]);
-        for (int c = 0; c < OUT; ++c) ys[(size_t)i * OUT + c] = (float)((Y[(size_t)i * OUT + c] - m->my[c]) / m->sy[c]);
+        for (int c = 0; c < IN; ++c) xs[(size_t)i * IN + c] = (float)((X[(size_t)i * IN + c] - m->sd.mx[c]) / m->sd.sx[c]);
+        for (int c = 0; c < OUT; ++c) ys[(size_t)i * OUT + c] = (float)((Y[(size_t)i * OUT + c] - m->sd.my[c]) / m->sd.sy[c]);
     }
     MCU(cudaMemcpyAsync(m->X, xs.data(), xs.size() * sizeof(float), cudaMemcpyHostToDevice, m->st));
     MCU(cudaMemcpyAsync(m->T, ys.data(), ys.size() * sizeof(float), cudaMemcpyHostToDevice, m->st));
@@ -593,35 +644,28 @@ tdpd_status tdpd_mlp_predict(tdpd_mlp *m, int n, const float *X, float *mean, fl
 {
     if (!m || n < 1 || !X || !mean) return mfail(TDPD_EINVAL, "tdpd_mlp_predict: bad arguments");
     if (!m->have_data) return mfail(TDPD_ESTATE, "tdpd_mlp_predict: no standardisation (set data first)");
-    // prediction buffers: reuse the training buffers when large enough
-    float *dX = nullptr, *dY = nullptr;
-    MCU(cudaMallocAsync((void **)&dX, (size_t)n * IN * sizeof(float), m->st));
-    MCU(cudaMallocAsync((void **)&dY, (size_t)m->members * n * OUT * sizeof(float), m->st));
-    std::vector<float> xs((size_t)n * IN), ys((size_t)m->members * n * OUT);
-    for (int i = 0; i < n; ++i)
-        for (int c = 0; c < IN; ++c) xs[(size_t)i * IN + c] = (float)((X[(size_t)i * IN + c] - m->mx[c]) / m->sx[c]);
-    MCU(cudaMemcpyAsync(dX, xs.data(), xs.size() * sizeof(float), cudaMemcpyHostToDevice, m->st));
-    k_mlp_fwd<<<dim3((n + CH - 1) / CH, m->members), TPB, 0, m->st>>>(m->params, dX, n, dY);
+    const size_t N = (size_t)n, in = N * IN, ens = 2 * N * OUT, each = (size_t)m->members * N * OUT;
+    const size_t need = in + ens + each;
+    // a call beyond the kept workspace allocates for itself
+    const bool keep = need <= PRED_KEEP;
+    float *d = nullptr;
+    if (keep) {
+        tdpd_status rc = pred_workspace(m, need);
+        if (rc) return rc;
+        d = m->pred;
+    } else {
+        MCU(cudaMallocAsync((void **)&d, need * sizeof(float), m->st));
+    }
+    float *dmean = d + in, *drel = dmean + N * OUT, *dY = drel + N * OUT;
+    MCU(cudaMemcpyAsync(d, X, in * sizeof(float), cudaMemcpyHostToDevice, m->st));
+    k_mlp_fwd<<<dim3((n + CH - 1) / CH, m->members), TPB, 0, m->st>>>(m->params, d, m->sd, n, dY);
+    launch_pdl(k_mlp_stats, (unsigned)((N * OUT + TPB - 1) / TPB), TPB, m->st, dY, m->sd, m->members, n, dmean, drel);
     MCU(cudaGetLastError());
-    MCU(cudaMemcpyAsync(ys.data(), dY, ys.size() * sizeof(float), cudaMemcpyDeviceToHost, m->st));
-    MCU(cudaFreeAsync(dX, m->st));
-    MCU(cudaFreeAsync(dY, m->st));
+    MCU(cudaMemcpyAsync(mean, dmean, N * OUT * sizeof(float), cudaMemcpyDeviceToHost, m->st));
+    if (rel_spread) MCU(cudaMemcpyAsync(rel_spread, drel, N * OUT * sizeof(float), cudaMemcpyDeviceToHost, m->st));
+    if (member_out) MCU(cudaMemcpyAsync(member_out, dY, each * sizeof(float), cudaMemcpyDeviceToHost, m->st));
+    if (!keep) MCU(cudaFreeAsync(d, m->st));
     MCU(cudaStreamSynchronize(m->st));
-    const int M = m->members;
-    for (int i = 0; i < n; ++i)
-        for (int c = 0; c < OUT; ++c) {
-            double s = 0.0, s2 = 0.0;
-            for (int k = 0; k < M; ++k) {
-                const double y = ys[((size_t)k * n + i) * OUT + c] * m->sy[c] + m->my[c];
-                if (member_out) member_out[((size_t)k * n + i) * OUT + c] = (float)y;
-                s += y;
-                s2 += y * y;
-            }
-            const double mu = s / M;
-            const double var = M > 1 ? std::max(0.0, (s2 - M * mu * mu) / (M - 1)) : 0.0;
-            mean[(size_t)i * OUT + c] = (float)mu;
-            if (rel_spread) rel_spread[(size_t)i * OUT + c] = (float)(std::sqrt(var) / std::max(std::fabs(mu), 1e-30));
-        }
     return TDPD_OK;
 }
 
@@ -630,10 +674,8 @@ void tdpd_mlp_destroy(tdpd_mlp *m)
     if (!m) return;
     cudaStreamSynchronize(m->st);
     free_data(m);
-    cudaFree(m->params);
-    cudaFree(m->m);
-    cudaFree(m->v);
-    cudaFree(m->grad);
+    if (m->pred_own) cudaFree(m->pred_own);
+    cudaFree(m->base);
     cudaStreamDestroy(m->st);
     delete m;
 }
