@@ -458,6 +458,48 @@ MemArgs mem_args(tdpd_sys *s, int ref_in, int inc)
     return m;
 }
 
+// List mode with one or two species (and no random flux): the pair kernel
+// (its one- and two-species forms) builds the lists of rebuilding replicas
+// itself; the forms for more species and for the random flux read striped lists
+// (list_striped.cuh) that a kernel of their own builds before them.
+bool pair_builds_lists(const tdpd_sys *s)
+{
+    if (!s->use_list || s->ns > 2) return false;
+    for (const HostRep &R : s->reps)
+        if (R.qr_ms > 0.0f) return false;
+    return true;
+}
+
+bool striped_lists(const tdpd_sys *s) { return s->use_list && !pair_builds_lists(s); }
+
+// Rounds per warp of the kernels on striped lists (a power of two up to the
+// lanes, so that a warp holds at most 32 particles): as many as leave the GPU
+// enough warps to fill it about one and a half times (152 SMs x 16 resident
+// warps), since a warp's set-up is paid once for all its rounds.
+int pair_klog(int N, int lanes)
+{
+    constexpr long WARPS = 152 * 16 * 3 / 2;
+    int k = 0;
+    while ((1 << (k + 1)) <= lanes && (long)N * lanes / 32 >= WARPS << (k + 1)) ++k;
+    return k;
+}
+
+// Entries a list can hold: 1.5 x the longest plus 16; a striped list read by
+// several lanes a little more, in whole blocks of the lanes.
+int list_capacity(int longest, bool striped, int lanes)
+{
+    const int cap = striped && lanes > 1 ? longest * 2 + 16 + 4 * lanes : longest * 3 / 2 + 16;
+    const int unit = striped ? std::max(8, lanes) : 8;
+    return (cap + unit - 1) / unit * unit;
+}
+
+// Ints of the list array: cap blocks of 32 lanes' entries per warp, or cap /
+// lanes blocks of 32 entries per 32 / lanes particles.
+size_t list_ints(int N, bool striped, int lanes, int cap)
+{
+    return ((size_t)N * lanes + 31) / 32 * 32 * (size_t)(striped ? cap / lanes : cap);
+}
+
 // disp_next: where list mode records the displacements of the next positions
 // build_rb (list mode): the replicas whose lanes build their lists inside
 // the pair kernel first (a rebuild step)
@@ -470,8 +512,10 @@ PairArgs pair_args(tdpd_sys *s, const Buffers &b, int integrate, int *tile_sum, 
     a.cellrank = s->cellrank; a.err = s->errw; a.quar = s->quar; a.step_ctr = s->step_ctr; a.n = s->N; a.ns = s->ns;
     a.integrate = integrate;
     a.lpp = s->lpp;
+    a.klog = pair_klog(s->N, s->lpp);
     a.std_exp = 1;
     for (const HostRep &R : s->reps) {
+        a.nt = std::max(a.nt, (int)R.cfg.n_types);
         if (R.qr_ms > 0.0f) a.qr = 1;
         if (!(R.cfg.s_f == 2.0f && R.cfg.s_c == 2.0f)) a.std_exp = 0;
     }
@@ -500,6 +544,7 @@ ListArgs list_args(tdpd_sys *s, const Buffers &b, const uint32_t *rb, int cap)
     l.m2 = 1;
     for (const HostRep &R : s->reps) l.m2 = l.m2 && R.m == 2;
     l.half = s->half ? 1 : 0;
+    l.striped = striped_lists(s) ? 1 : 0;
     return l;
 }
 
@@ -518,17 +563,6 @@ Quarantine quarantine(tdpd_sys *s)
 // kernel's launch; more replicas keep the separate kernel.
 constexpr int DECIDE_INLINE_MAX = 16;
 bool inline_decide(const tdpd_sys *s) { return (int)s->reps.size() <= DECIDE_INLINE_MAX; }
-
-// List mode with one or two species (and no random flux): the pair kernel
-// (its one- and two-species forms) builds the lists of rebuilding replicas
-// itself; otherwise k_list_build runs before it.
-bool pair_builds_lists(const tdpd_sys *s)
-{
-    if (!s->use_list || s->ns > 2) return false;
-    for (const HostRep &R : s->reps)
-        if (R.qr_ms > 0.0f) return false;
-    return true;
-}
 
 // The one-cluster sort of step p (reading buffer p): its decision reads the
 // maxima of the last epilogue, like k_bin_next's inline decision.
@@ -833,20 +867,17 @@ tdpd_status init_state(tdpd_sys *s)
 // mode (idempotent apart from the next binning's counters) for each choice,
 // then rebuild the state with the winner.
 // Size the neighbour lists of the current lane count from a counting pass
-// over the sorted state in buffer 1 (capacity: 1.5 x the longest lane list,
-// plus 16), allocate them and build them.
+// over the sorted state in buffer 1 (list_capacity), allocate them and build them.
 tdpd_status prepare_list(tdpd_sys *s)
 {
     cudaStream_t st = exec_stream(s);
-    const size_t lanes = (size_t)s->N * s->lpp;
+    const bool striped = striped_lists(s);
     launch_list_build(list_args(s, s->buf[1], s->rb_all, 0), st);
-    std::vector<int> cnt(lanes);
-    CU(cudaMemcpyAsync(cnt.data(), s->nlc, sizeof(int) * lanes, cudaMemcpyDeviceToHost, st));
+    std::vector<int> cnt((size_t)s->N * (striped ? 1 : s->lpp));
+    CU(cudaMemcpyAsync(cnt.data(), s->nlc, sizeof(int) * cnt.size(), cudaMemcpyDeviceToHost, st));
     CU(cudaStreamSynchronize(st));
-    int mx = 0;
-    for (int c : cnt) mx = std::max(mx, c);
-    const int cap = (mx * 3 / 2 + 16 + 7) / 8 * 8;
-    const size_t need = (lanes + 31) / 32 * 32 * (size_t)cap;
+    const int cap = list_capacity(*std::max_element(cnt.begin(), cnt.end()), striped, s->lpp);
+    const size_t need = list_ints(s->N, striped, s->lpp, cap);
     if (need > s->nl_ints) {
         if (s->nl) CU(cudaFree(s->nl));
         s->nl = nullptr;
@@ -907,7 +938,7 @@ tdpd_status autotune(tdpd_sys *s)
     for (int mode : modes) {
         for (int lpp = 1; lpp <= 32; lpp *= 2) {
             if (s->lanes_fixed > 0 && lpp != s->lanes_fixed) continue;
-            if (s->lanes_fixed == 0 && lpp > 1 && (long)s->N * lpp > 4000000L) break;
+            if (s->lanes_fixed == 0 && lpp > (striped_lists(s) ? 8 : 1) && (long)s->N * lpp > 4000000L) break;
             s->lpp = lpp;
             s->half = mode == 2;
             tdpd_status rc;
@@ -1340,7 +1371,8 @@ tdpd_status commit(tdpd_sys *s)
             s->h_chunks.push_back(make_int4((int)r, b0 + k, b0 + std::min(n, k + OBS_CHUNK), 0));
     }
     // lanes per particle: enough threads to fill the GPU (~300k resident)
-    s->lpp = 1;
+    // (striped lists: eight, whose entries share sectors)
+    s->lpp = striped_lists(s) ? 8 : 1;
     while (s->lpp < 8 && (long)N * s->lpp < 300000) s->lpp *= 2;
     s->n_rbc = (int)s->h_rbcs.size();
     s->all_lagged = s->n_rbc > 0;
@@ -1964,7 +1996,7 @@ tdpd_status config_hash(tdpd_sys *s, uint64_t *out)
 }
 
 // (device pointer, bytes) of every saved array, in file order
-std::vector<std::pair<void *, size_t>> ckp_arrays(tdpd_sys *s, int parity, size_t nl_ints)
+std::vector<std::pair<void *, size_t>> ckp_arrays(tdpd_sys *s, int parity, size_t nl_ints, uint32_t version)
 {
     const size_t N = (size_t)s->N, ns = (size_t)s->ns, nr = s->reps.size(), nb = (size_t)s->n_rbc;
     const Buffers &B = s->buf[parity];
@@ -1988,9 +2020,12 @@ std::vector<std::pair<void *, size_t>> ckp_arrays(tdpd_sys *s, int parity, size_
         v.push_back({s->disp[0], 4 * nr});
         v.push_back({s->disp[1], 4 * nr});
         v.push_back({s->builds, 4 * nr});
-        v.push_back({s->nlc, 4 * N * (size_t)s->lpp});
+        // (striped lists are not read from a version 2 file, which holds one
+        // list per lane: null, and the next step rebuilds them)
+        const bool striped = striped_lists(s), skip = striped && version < 3;
+        v.push_back({skip ? nullptr : s->nlc, 4 * N * (striped && !skip ? 1 : (size_t)s->lpp)});
         v.push_back({s->xb, 16 * N});
-        v.push_back({s->nl, 4 * nl_ints});
+        v.push_back({skip ? nullptr : s->nl, 4 * nl_ints});
     }
     if (nb) {
         v.push_back({s->mx, 16 * N});
@@ -2006,8 +2041,11 @@ std::vector<std::pair<void *, size_t>> ckp_arrays(tdpd_sys *s, int parity, size_
 
 size_t nl_used_ints(const tdpd_sys *s)
 {
-    return s->use_list ? ((size_t)s->N * s->lpp + 31) / 32 * 32 * (size_t)s->nl_cap : 0;
+    return s->use_list ? list_ints(s->N, striped_lists(s), s->lpp, s->nl_cap) : 0;
 }
+
+// 2: list mode also saves the other buffer; 3: the same with striped lists
+uint32_t ckp_version(const tdpd_sys *s) { return striped_lists(s) ? 3 : 2; }
 
 tdpd_status tdpd_save(tdpd_sys *s, const char *path)
 {
@@ -2016,7 +2054,7 @@ tdpd_status tdpd_save(tdpd_sys *s, const char *path)
     if (!path) return fail(s, TDPD_EINVAL, "null path");
     CkpHeader H{};
     std::memcpy(H.magic, CKP_MAGIC, 8);
-    H.version = 2;     // 2: list mode also saves the other buffer
+    H.version = ckp_version(s);
     H.N = s->N; H.NC = s->NC; H.ns = s->ns; H.n_rep = (int)s->reps.size(); H.n_rbc = s->n_rbc;
     H.lpp = s->lpp; H.use_list = s->use_list ? (s->half ? 2 : 1) : 0; H.nl_cap = s->nl_cap; H.parity = s->parity;
     H.n_tiles = s->n_tiles; H.step = s->step;
@@ -2027,7 +2065,7 @@ tdpd_status tdpd_save(tdpd_sys *s, const char *path)
     if (!f) return fail(s, TDPD_EINVAL, "cannot open %s for writing", path);
     bool ok = std::fwrite(&H, sizeof H, 1, f) == 1;
     std::vector<unsigned char> host;
-    for (const auto &a : ckp_arrays(s, s->parity, H.nl_ints)) {
+    for (const auto &a : ckp_arrays(s, s->parity, H.nl_ints, H.version)) {
         if (!ok) break;
         host.resize(a.second);
         cudaError_t e = cudaMemcpy(host.data(), a.first, a.second, cudaMemcpyDeviceToHost);
@@ -2050,14 +2088,15 @@ tdpd_status tdpd_load(tdpd_sys *s, const char *path)
     FILE *f = std::fopen(path, "rb");
     if (!f) return fail(s, TDPD_EINVAL, "cannot open %s", path);
     CkpHeader H{};
-    if (std::fread(&H, sizeof H, 1, f) != 1 || std::memcmp(H.magic, CKP_MAGIC, 8) != 0 || H.version != 2) {
+    if (std::fread(&H, sizeof H, 1, f) != 1 || std::memcmp(H.magic, CKP_MAGIC, 8) != 0 ||
+        (H.version != 2 && H.version != 3)) {
         std::fclose(f);
         return fail(s, TDPD_EINVAL, "%s is not a checkpoint of this library", path);
     }
     uint64_t h = 0;
     if ((rc = config_hash(s, &h))) { std::fclose(f); return rc; }
     if (H.N != s->N || H.NC != s->NC || H.ns != s->ns || H.n_rep != (int)s->reps.size() || H.n_rbc != s->n_rbc ||
-        (H.use_list != 0) != s->use_list || H.n_tiles != s->n_tiles || H.cfg_hash != h) {
+        (H.use_list != 0) != s->use_list || H.n_tiles != s->n_tiles || H.cfg_hash != h || H.version > ckp_version(s)) {
         std::fclose(f);
         return fail(s, TDPD_EINVAL, "checkpoint of another configuration (particles, cells, species, replicas, "
                                     "membranes, list mode or parameters differ)");
@@ -2077,14 +2116,19 @@ tdpd_status tdpd_load(tdpd_sys *s, const char *path)
         std::fclose(f);
         return fail(s, TDPD_EINVAL, "corrupt checkpoint header");
     }
-    // the list layout follows the capacity of the saved run
-    const bool recapture = s->use_list && H.nl_cap != s->nl_cap;
+    // the list layout follows the capacity of the saved run (lists of the other
+    // layout are skipped, and the capacity stays)
+    const bool skip = s->use_list && H.version < ckp_version(s);
+    const bool recapture = s->use_list && !skip && H.nl_cap != s->nl_cap;
     if (s->use_list) {
-        const size_t need = ((size_t)s->N * s->lpp + 31) / 32 * 32 * (size_t)H.nl_cap;
-        if (H.nl_cap <= 0 || need != H.nl_ints) {
+        const size_t need = list_ints(s->N, H.version >= 3, s->lpp, H.nl_cap);
+        if (H.nl_cap <= 0 || (H.version >= 3 && H.nl_cap % s->lpp != 0) || need != H.nl_ints) {
             std::fclose(f);
             return fail(s, TDPD_EINVAL, "corrupt checkpoint header");
         }
+    }
+    if (s->use_list && !skip) {
+        const size_t need = H.nl_ints;
         if (need > s->nl_ints) {
             CU(cudaStreamSynchronize(exec_stream(s)));
             if (s->nl) CU(cudaFree(s->nl));
@@ -2102,9 +2146,10 @@ tdpd_status tdpd_load(tdpd_sys *s, const char *path)
     CU(cudaStreamSynchronize(exec_stream(s)));
     std::vector<unsigned char> host;
     bool ok = true;
-    for (const auto &a : ckp_arrays(s, H.parity, H.nl_ints)) {
+    for (const auto &a : ckp_arrays(s, H.parity, H.nl_ints, H.version)) {
         host.resize(a.second);
         if (a.second && std::fread(host.data(), 1, a.second, f) != a.second) { ok = false; break; }
+        if (!a.first) continue;
         cudaError_t e = cudaMemcpy(a.first, host.data(), a.second, cudaMemcpyHostToDevice);
         if (e != cudaSuccess) {
             std::fclose(f);
@@ -2113,6 +2158,12 @@ tdpd_status tdpd_load(tdpd_sys *s, const char *path)
     }
     std::fclose(f);
     if (!ok) return fail(s, TDPD_EINVAL, "%s is truncated; the handle's state is undefined until the next load", path);
+    if (skip) {
+        // a displacement beyond any skin: every replica rebuilds at the next step
+        const std::vector<float> far(s->reps.size(), 1e30f);
+        for (int k = 0; k < 2; ++k)
+            CU(cudaMemcpy(s->disp[k], far.data(), sizeof(float) * far.size(), cudaMemcpyHostToDevice));
+    }
     s->parity = H.parity;
     s->step = H.step;
     if (recapture && (rc = capture_graphs(s))) return rc;

@@ -14,16 +14,21 @@
 // Layout: entry k of lane l of warp w at nl[(w * cap + k) * 32 + l], so the
 // 32 lanes of a warp read one 128-byte line per entry.
 //
-// k_list_build builds the lists of a loaded state; on a rebuild step the pair
-// kernel's one- and two-species forms build their own lanes' lists
-// (list_lane.cuh), and k_list_build runs only for the other forms.
+// k_list_build counts the entries at commit; on a rebuild step and for a loaded
+// state the pair kernel's one- and two-species forms build their own lanes' lists
+// (list_lane.cuh). The kernels for more species and for the random flux read
+// lists of another layout (list_striped.cuh), one per particle, which
+// k_list_build_striped builds before them.
 #include <algorithm>
 #include <type_traits>
 
 #include "launch.h"
 #include "list_lane.cuh"
+#include "list_striped.cuh"
 
 namespace tdpd {
+
+constexpr int STRIPED_SPLIT_MAX = 60000;
 
 __global__ void k_rebuild_decide(const uint32_t *__restrict__ disp, uint32_t *disp_clear, uint32_t *rb,
                                  const RepParams *__restrict__ reps, int n_rep, int force, uint32_t *step_ctr,
@@ -122,6 +127,68 @@ __global__ void __launch_bounds__(128) k_list_build(ListArgs A)
     build_lane<LPP, M, HALF>(A, gt, i, sub, pi, rep);
 }
 
+// The striped lists of the kernels with more than two species, B threads per
+// particle (a power of two): thread s takes the s-th of B consecutive parts of
+// the stencil's rows, counts its entries, and writes them after those of the
+// threads before it, so a list has the same order for every B. One thread walks
+// its rows once; several (small systems, where a thread per particle leaves the
+// GPU idle) walk them twice.
+template <int M, bool HALF, int B>
+__global__ void __launch_bounds__(128) k_list_build_striped(ListArgs A)
+{
+    pdl_enter();
+    if (!A.rb[A.n_rep]) return;                       // no replica rebuilds
+    const int gt = blockIdx.x * blockDim.x + threadIdx.x;
+    const int i = gt / B, sub = gt % B;
+    const bool valid = i < A.n;
+    const float4 pi = A.pos[valid ? i : 0];
+    const int rep = wbits(A.vel[valid ? i : 0].w);
+    bool need = valid && A.rb[rep] != 0u;
+    if (need && A.quar && A.quar[rep]) {              // quarantined: an empty list
+        if (sub == 0) A.nlc[i] = 0;
+        need = false;
+    }
+    const RepParams &P = A.reps[rep];
+    const int m = M > 0 ? M : P.m_stencil, nrow = (2 * m + 1) * (2 * m + 1);
+    const int first = HALF ? nrow / 2 : 0, rows = nrow - first;
+    const int r0 = first + rows * sub / B, r1 = need ? first + rows * (sub + 1) / B : r0;
+    int e = 0, total = 0;
+    if (B > 1) {
+        int c = 0;
+        visit_rows<M, HALF>(P, A.pos, A.cell_start, i, r0, r1, 1, pi, [&](const bool (&ok)[4], int) {
+            c += (int)ok[0] + (int)ok[1] + (int)ok[2] + (int)ok[3];
+        });
+        int x = c;
+#pragma unroll
+        for (int o = 1; o < B; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, x, o, B);
+            if (sub >= o) x += v;
+        }
+        e = x - c;
+        total = __shfl_sync(0xffffffffu, x, B - 1, B);
+    }
+    if (B == 1 || A.cap > 0) {
+        const int L = A.lpp, cap = A.cap;
+        int *list = A.nl + striped_row(i, L, cap / L);
+        int at = striped_off(e, L);
+        visit_rows<M, HALF>(P, A.pos, A.cell_start, i, r0, r1, 1, pi, [&](const bool (&ok)[4], int j0) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (ok[u]) {
+                    if (e < cap) list[at] = j0 + u;
+                    ++e;
+                    at += (e & (L - 1)) ? 1 : 33 - L;
+                }
+        });
+        if (B == 1) total = e;
+    }
+    if (need && sub == 0) {
+        A.nlc[i] = A.cap > 0 ? min(total, A.cap) : total;
+        if (A.cap > 0 && total > A.cap) atomicOr(A.err + rep, 2u);
+        A.xb[i] = pi;
+    }
+}
+
 void launch_rebuild_decide(const uint32_t *disp, uint32_t *disp_clear, uint32_t *rb, const RepParams *reps,
                            int n_rep, int force, uint32_t *step_ctr, uint32_t *builds, cudaStream_t st)
 {
@@ -159,9 +226,29 @@ static void launch_list_build_h(const ListArgs &a, int g, cudaStream_t st)
     }
 }
 
+template <int M, bool HALF>
+static void launch_striped(const ListArgs &a, cudaStream_t st)
+{
+    // eight threads per particle up to the particles that fill the GPU alone
+    if (a.n <= STRIPED_SPLIT_MAX)
+        launch_pdl(k_list_build_striped<M, HALF, 8>, (int)((8L * a.n + 127) / 128), 128, st, a);
+    else
+        launch_pdl(k_list_build_striped<M, HALF, 1>, (a.n + 127) / 128, 128, st, a);
+}
+
 void launch_list_build(const ListArgs &a, cudaStream_t st)
 {
     if (a.n <= 0) return;
+    if (a.striped) {
+        if (a.m2) {
+            if (a.half) launch_striped<2, true>(a, st);
+            else launch_striped<2, false>(a, st);
+        } else {
+            if (a.half) launch_striped<0, true>(a, st);
+            else launch_striped<0, false>(a, st);
+        }
+        return;
+    }
     const int g = (int)(((long)a.n * a.lpp + 127) / 128);
     if (a.half) launch_list_build_h<true>(a, g, st);
     else launch_list_build_h<false>(a, g, st);

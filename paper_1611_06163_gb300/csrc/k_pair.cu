@@ -1,6 +1,7 @@
 // Instantiation of the pair kernels with exponents read per replica, the
 // half shell's finishing pass, and the dispatch (the kernels themselves are
-// in k_pair_impl.cuh).
+// in k_pair_impl.cuh; those for more than two species and for the random flux in
+// k_pair_multi.cuh, instantiated in k_pair_multi.cu and k_pair_flux.cu).
 #include "k_pair_impl.cuh"
 
 namespace tdpd {
@@ -8,10 +9,9 @@ namespace tdpd {
 void launch_pair_finish(const PairArgs &a, cudaStream_t st)
 {
     const int g = (a.n + 255) / 256;
-    switch (a.qr ? 0 : a.ns) {
+    switch (a.ns) {
     case 1: launch_pdl(k_pair_finish<1>, g, 256, st, a); break;
     case 2: launch_pdl(k_pair_finish<2>, g, 256, st, a); break;
-    case 10: launch_pdl(k_pair_finish<10>, g, 256, st, a); break;
     default: launch_pdl(k_pair_finish<0>, g, 256, st, a); break;
     }
 }
@@ -21,17 +21,18 @@ void launch_pair(const PairArgs &a, cudaStream_t st, int part)
     if (a.n <= 0) return;
     if (a.std_exp && !a.qr && (a.ns == 1 || a.ns == 2)) {
         launch_pair_std(a, st, part);
-    } else if (a.qr) {
-        // the random flux lives in the general kernel only
-        if (a.nl) launch_ns<0, true, false>(a, st, part);
-        else launch_ns<0, false, false>(a, st, part);
-    } else if (a.nl) {
-        switch (a.ns) {
-        case 1: launch_ns<1, true, false>(a, st, part); break;
-        case 2: launch_ns<2, true, false>(a, st, part); break;
-        case 10: launch_ns<10, true, false>(a, st, part); break;     // the paper's ten-species case
-        default: launch_ns<0, true, false>(a, st, part); break;
+    } else if (a.nl && (a.qr || a.ns > 2)) {
+        if (part & PAIR_WALK) {
+            if (a.qr) launch_pair_flux(a, st);
+            else launch_pair_multi(a, st);
         }
+        if (a.half && (part & PAIR_FINISH)) launch_pair_finish(a, st);
+    } else if (a.nl) {
+        if (a.ns == 1) launch_ns<1, true, false>(a, st, part);
+        else launch_ns<2, true, false>(a, st, part);
+    } else if (a.qr) {
+        // cell mode: the random flux lives in the general kernel only
+        launch_ns<0, false, false>(a, st, part);
     } else {
         switch (a.ns) {
         case 1: launch_ns<1, false, false>(a, st, part); break;

@@ -9,38 +9,34 @@
 
 namespace tdpd {
 
-// The list of one pair lane (particle i, lane sub of LPP, thread gt of the
-// pair kernel's layout) over the cell stencil, its count in nlc and, for lane
-// 0, the build position xb[i]. M: the stencil half-width when it is known at
-// compile time (2, the default cell size), else 0 (read per replica). Used by
-// k_list_build and, on rebuild steps, by the pair kernel for its own lanes.
+// The candidates of particle i over the rows r0, r0 + dr, ... < r1 of its cell
+// stencil, in row order and slot order within a row: hit(ok, j0) for four
+// candidate slots j0 .. j0 + 3 at a time, ok[u] set where slot j0 + u holds a
+// partner within rlist. M: the stencil half-width when it is known at compile
+// time (2, the default cell size), else 0 (read per replica).
 //
-// HALF: only the upper half of the stencil, so that every unordered pair is
-// listed once. A cell's offset (dx, dy, dz) from particle i's cell has one
-// representative in [-m, m]^3 (a periodic axis holds at least 2m + 1 cells),
-// and the pair belongs to the side from which that offset is upper: rows
-// with dz > 0, or dz = 0 and dy > 0 (the rows after the home row), and in
-// the home row the cells with dx > 0 and, in i's own cell, the slots after
-// i. Cells of a row are consecutive slots, so the home row's upper part is
-// the slot range after i up to the row's end, plus the segment that wraps
-// around to the right.
-template <int LPP, int M, bool HALF = false>
-__device__ __forceinline__ void build_lane(const ListArgs &A, int gt, int i, int sub, float4 pi, int rep)
+// HALF: only the upper half of the stencil (rows from (2m+1)^2 / 2 on), so that
+// every unordered pair is listed once. A cell's offset (dx, dy, dz) from particle
+// i's cell has one representative in [-m, m]^3 (a periodic axis holds at least
+// 2m + 1 cells), and the pair belongs to the side from which that offset is
+// upper: rows with dz > 0, or dz = 0 and dy > 0 (the rows after the home row),
+// and in the home row the cells with dx > 0 and, in i's own cell, the slots after
+// i. Cells of a row are consecutive slots, so the home row's upper part is the
+// slot range after i up to the row's end, plus the segment that wraps around to
+// the right.
+template <int M, bool HALF, class Hit>
+__device__ __forceinline__ void visit_rows(const RepParams &P, const float4 *pos, const int *cell_start, int i,
+                                           int r0, int r1, int dr, float4 pi, Hit &&hit)
 {
-    const RepParams &P = A.reps[rep];
-    const int m = M > 0 ? M : P.m_stencil, width = 2 * m + 1, nrow = width * width;
+    const int m = M > 0 ? M : P.m_stencil, width = 2 * m + 1;
     const int cx = cell_coord(pi.x, P.cell_scale[0], P.nc[0]);
     const int cy = cell_coord(pi.y, P.cell_scale[1], P.nc[1]);
     const int cz = cell_coord(pi.z, P.cell_scale[2], P.nc[2]);
     const float oy = pi.y - (float)cy * P.h[1], oz = pi.z - (float)cz * P.h[2];
     const float eps = 1e-4f * fmaxf(P.h[0], fmaxf(P.h[1], P.h[2]));
     const float rl2 = P.rlist2;
-    int *out = A.nl + (size_t)(gt >> 5) * A.cap * 32 + (gt & 31);   // next entry
-    const int cap = A.cap;
-    int c = 0;
-    // the row's candidates, four per trip with their loads in flight together,
-    // appended in slot order (the capacity test once per trip while four more
-    // entries fit); SELF: the home row, which holds particle i itself
+    // the row's candidates, four per trip with their loads in flight together;
+    // SELF: the home row, which holds particle i itself
     auto walk = [&](const RowSeg &g, auto self) {
         constexpr bool SELF = decltype(self)::value;
         const float py = pi.y + g.sy, pz = pi.z + g.sz;
@@ -51,39 +47,21 @@ __device__ __forceinline__ void build_lane(const ListArgs &A, int gt, int i, int
             for (int j0 = g.jb[sg]; j0 < je; j0 += 4) {
                 float4 pj[4];
 #pragma unroll
-                for (int u = 0; u < 4; ++u) pj[u] = j0 + u < je ? A.pos[j0 + u] : make_float4(1e30f, 0.f, 0.f, 0.f);
+                for (int u = 0; u < 4; ++u) pj[u] = j0 + u < je ? pos[j0 + u] : make_float4(1e30f, 0.f, 0.f, 0.f);
                 bool ok[4];
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
                     const float dx = px - pj[u].x, dy = py - pj[u].y, dz = pz - pj[u].z;
                     ok[u] = dx * dx + dy * dy + dz * dz < rl2 && (!SELF || j0 + u != i);
                 }
-                if (c + 4 <= cap) {
-#pragma unroll
-                    for (int u = 0; u < 4; ++u)
-                        if (ok[u]) {
-                            *out = j0 + u;
-                            out += 32;
-                            ++c;
-                        }
-                } else {
-#pragma unroll
-                    for (int u = 0; u < 4; ++u)
-                        if (ok[u]) {
-                            if (c < cap) {
-                                *out = j0 + u;
-                                out += 32;
-                            }
-                            ++c;
-                        }
-                }
+                hit(ok, j0);
             }
         }
     };
-    for (int row = (HALF ? nrow / 2 : 0) + sub; row < nrow; row += LPP) {
+    for (int row = r0; row < r1; row += dr) {
         const int dy = row % width - m, dz = row / width - m;
         RowSeg g = {{0, 0}, {0, 0}, 0.f, 0.f, 0.f};
-        if (!stencil_row_d(P, A.cell_start, pi, cx, cy, cz, dy, dz, m, oy, oz, eps, rl2 * 1.0002f, g)) continue;
+        if (!stencil_row_d(P, cell_start, pi, cx, cy, cz, dy, dz, m, oy, oz, eps, rl2 * 1.0002f, g)) continue;
         if (dy == 0 && dz == 0) {
             if (HALF) {
                 // the home row from the slot after i; a segment that wraps
@@ -96,6 +74,43 @@ __device__ __forceinline__ void build_lane(const ListArgs &A, int gt, int i, int
             walk(g, std::false_type{});
         }
     }
+}
+
+// The list of one pair lane (particle i, lane sub of LPP, thread gt of the pair
+// kernel's layout), its count in nlc and, for lane 0, the build position xb[i].
+// Used by k_list_build and, on rebuild steps, by the pair kernel for its own
+// lanes.
+template <int LPP, int M, bool HALF = false>
+__device__ __forceinline__ void build_lane(const ListArgs &A, int gt, int i, int sub, float4 pi, int rep)
+{
+    const RepParams &P = A.reps[rep];
+    const int m = M > 0 ? M : P.m_stencil, nrow = (2 * m + 1) * (2 * m + 1);
+    int *out = A.nl + (size_t)(gt >> 5) * A.cap * 32 + (gt & 31);   // next entry
+    const int cap = A.cap;
+    int c = 0;
+    // appended in order (the capacity test once per four while they fit)
+    visit_rows<M, HALF>(P, A.pos, A.cell_start, i, (HALF ? nrow / 2 : 0) + sub, nrow, LPP, pi,
+                        [&](const bool (&ok)[4], int j0) {
+        if (c + 4 <= cap) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (ok[u]) {
+                    *out = j0 + u;
+                    out += 32;
+                    ++c;
+                }
+        } else {
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (ok[u]) {
+                    if (c < cap) {
+                        *out = j0 + u;
+                        out += 32;
+                    }
+                    ++c;
+                }
+        }
+    });
     A.nlc[gt] = A.cap > 0 ? min(c, A.cap) : c;
     if (A.cap > 0 && c > A.cap) atomicOr(A.err + rep, 2u);
     if (sub == 0) A.xb[i] = pi;

@@ -485,7 +485,7 @@ tdpd_status alloc_data(tdpd_mlp *m, int n)
 // the handle, more are allocated once. (Two allocations and their release on every
 // call, the standardisation and the ensemble statistics on the host took 250 us of
 // a call that ranks 2048 points with five members.)
-constexpr size_t PRED_MIN = (size_t)1 << 17, PRED_KEEP = (size_t)1 << 22;
+constexpr size_t PRED_MIN = (size_t)1 << 16, PRED_KEEP = (size_t)1 << 22;
 tdpd_status pred_workspace(tdpd_mlp *m, size_t need)
 {
     if (need <= m->pred_floats) return TDPD_OK;
