@@ -20,7 +20,6 @@
 // lists of another layout (list_striped.cuh), one per particle, which
 // k_list_build_striped builds before them.
 #include <algorithm>
-#include <type_traits>
 
 #include "launch.h"
 #include "list_lane.cuh"
@@ -155,7 +154,7 @@ __global__ void __launch_bounds__(128) k_list_build_striped(ListArgs A)
     int e = 0, total = 0;
     if (B > 1) {
         int c = 0;
-        visit_rows<M, HALF>(P, A.pos, A.cell_start, i, r0, r1, 1, pi, [&](const bool (&ok)[4], int) {
+        visit_rows<M, HALF, B == 1>(P, A.pos, A.cell_start, i, r0, r1, 1, pi, [&](const bool (&ok)[4], int) {
             c += (int)ok[0] + (int)ok[1] + (int)ok[2] + (int)ok[3];
         });
         int x = c;
@@ -167,11 +166,11 @@ __global__ void __launch_bounds__(128) k_list_build_striped(ListArgs A)
         e = x - c;
         total = __shfl_sync(0xffffffffu, x, B - 1, B);
     }
-    if (B == 1 || A.cap > 0) {
+    if (B == 1 ? need : A.cap > 0) {
         const int L = A.lpp, cap = A.cap;
         int *list = A.nl + striped_row(i, L, cap / L);
         int at = striped_off(e, L);
-        visit_rows<M, HALF>(P, A.pos, A.cell_start, i, r0, r1, 1, pi, [&](const bool (&ok)[4], int j0) {
+        visit_rows<M, HALF, B == 1>(P, A.pos, A.cell_start, i, r0, r1, 1, pi, [&](const bool (&ok)[4], int j0) {
 #pragma unroll
             for (int u = 0; u < 4; ++u)
                 if (ok[u]) {
