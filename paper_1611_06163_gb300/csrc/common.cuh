@@ -73,7 +73,7 @@ struct RbcDev {
     int tri_off;    // offset of its triangles (int[3 ntri]) in the triangle table
     int fan_off;    // offset of vertex 0's fan in the fan table
     int fan_stride; // fan entries per vertex: the mesh's largest degree
-    int pad_;
+    int edge_off;   // offset of its edges in the edge table
     double A0, V0;
     double kgA0, kvV0;  // k_g / A0, k_v / V0 (Eq. 14-15 coefficients per unit excess)
     double inv_nv;      // 1 / nv
@@ -92,10 +92,12 @@ struct RingEntry {
 // (entry v * fan_stride + l of its mesh), with the cyclic neighbours nb[l+1]
 // and nb[l-1] included: a lane reaches all its vertex indices with one
 // 32-byte load and no offset table. Entries past the degree have nb = -1.
+// end, opp: where k_membrane leaves the forces on v of the edges (v, nb[l]) and
+// (nb[l], nb[l+1]): the edge's index, v's place in its table entry << 29.
 struct __align__(16) FanEntry {
     int nb, edge, tri, across;
     int nb_next, nb_prev;
-    int pad0, pad1;
+    int end, opp;
 };
 
 // Programmatic dependent launch: let the next kernel in the stream begin

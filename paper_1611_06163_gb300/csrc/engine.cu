@@ -110,13 +110,12 @@ struct tdpd_sys {
     RbcDev *d_rbcs = nullptr;
     int *d_tri = nullptr;
     FanEntry *d_fan = nullptr;
+    int4 *d_edge = nullptr;
     float *d_a0j = nullptr;
     float2 *d_bond = nullptr;
     float4 *d_ref[2] = {nullptr, nullptr};
     double2 *d_av[2] = {nullptr, nullptr};   // (A, V) per membrane, written by step parity
     float2 *d_cgv[2] = {nullptr, nullptr};   // their constraint coefficients
-    bool all_lagged = false;                 // every membrane's K-Apply uses the previous totals
-    cudaEvent_t gathered = nullptr;          // lagged: K-Gather done on the side stream
     double *d_obs = nullptr, *d_obs_tot = nullptr;
     unsigned *d_obs_done = nullptr;
     float *d_in = nullptr;              // uploaded x, v, C of a loaded state (load order)
@@ -417,8 +416,6 @@ tdpd_status free_device(tdpd_sys *s)
     s->n_ev = 0;
     if (s->fork) cudaEventDestroy(s->fork);
     if (s->join) cudaEventDestroy(s->join);
-    if (s->gathered) cudaEventDestroy(s->gathered);
-    s->gathered = nullptr;
     if (s->side) cudaStreamDestroy(s->side);
     s->fork = s->join = nullptr;
     s->side = nullptr;
@@ -437,8 +434,8 @@ tdpd_status free_device(tdpd_sys *s)
     return TDPD_OK;
 }
 
-const char *const KERNEL_NAMES[] = {"scan",       "scatter_keys", "rank_gather", "mem_gather", "mem_forces",
-                                    "pair",       "decide",       "bin",         "list_build", "sort"};
+const char *const KERNEL_NAMES[] = {"scan", "scatter_keys", "rank_gather", "membrane", "pair",
+                                    "decide", "bin",        "list_build",  "sort"};
 
 // ref_in: which reference point buffer this evaluation reads; its K-Gather
 // writes the other one and the (A, V) buffer of the same index. inc: a step
@@ -449,10 +446,10 @@ MemArgs mem_args(tdpd_sys *s, int ref_in, int inc)
     const int q = 1 - ref_in;
     MemArgs m{};
     m.mx = s->mx; m.mv = s->mv; m.reps = s->d_reps; m.rbcs = s->d_rbcs;
-    m.tri = s->d_tri; m.fan = s->d_fan;
+    m.tri = s->d_tri; m.fan = s->d_fan; m.edge = s->d_edge;
     m.a0j = s->d_a0j; m.bond = s->d_bond; m.ref_in = s->d_ref[ref_in]; m.ref_out = s->d_ref[1 - ref_in];
-    m.av_out = s->d_av[q]; m.cgv_out = s->d_cgv[q]; m.cgv_seq = s->d_cgv[q];
-    m.cgv_lag = inc ? s->d_cgv[1 - q] : s->d_cgv[q];
+    m.av_out = s->d_av[q]; m.cgv_out = s->d_cgv[q];
+    m.cgv_lag = inc ? s->d_cgv[1 - q] : nullptr;
     m.fext = s->fext; m.n_rbc = s->n_rbc; m.max_nv = s->max_nv;
     m.mem_ctr = s->step_ctr + 1; m.q = q;
     return m;
@@ -594,15 +591,15 @@ std::vector<int> step_kernels(const tdpd_sys *s)
 {
     std::vector<int> k;
     if (s->use_list) {
-        if (s->sort_ctas) k = {9};
-        else if (inline_decide(s)) k = {7, 0, 1, 2};
-        else k = {6, 7, 0, 1, 2};
-        if (!pair_builds_lists(s)) k.push_back(8);
+        if (s->sort_ctas) k = {8};
+        else if (inline_decide(s)) k = {6, 0, 1, 2};
+        else k = {5, 6, 0, 1, 2};
+        if (!pair_builds_lists(s)) k.push_back(7);
     } else {
         k = {0, 1, 2};
     }
-    if (s->n_rbc) { k.push_back(3); k.push_back(4); }
-    k.push_back(5);
+    if (s->n_rbc) k.push_back(3);
+    k.push_back(4);
     return k;
 }
 
@@ -621,25 +618,14 @@ void enqueue_step(tdpd_sys *s, int p, cudaStream_t st, cudaEvent_t *ev = nullptr
     // needed only by the epilogue, which also writes the vertices' next
     // positions they read, so the branch joins just before the epilogue:
     // before k_pair_finish with the half shell (the branch then overlaps the
-    // sort and the pair walk), before the pair kernel otherwise. When every
-    // membrane's constraints are lagged, K-Apply goes first and K-Gather (for
-    // the next step) follows it on the branch. The timed step keeps one
-    // stream, so that the events bracket one kernel each.
+    // sort and the pair walk), before the pair kernel otherwise. The timed step
+    // keeps one stream, so that the events bracket one kernel each.
     const bool branch = s->n_rbc && !ev;
     if (branch) {
         cudaEventRecord(s->fork, st);
         cudaStreamWaitEvent(s->side, s->fork, 0);
-        const MemArgs m = mem_args(s, 1 - p, 1);
-        if (s->all_lagged) {
-            launch_mem_forces(m, s->side);
-            cudaEventRecord(s->join, s->side);
-            launch_mem_gather(m, s->side, true);
-            cudaEventRecord(s->gathered, s->side);
-        } else {
-            launch_mem_gather(m, s->side, false);
-            launch_mem_forces(m, s->side);
-            cudaEventRecord(s->join, s->side);
-        }
+        launch_membrane(mem_args(s, 1 - p, 1), s->side, false);
+        cudaEventRecord(s->join, s->side);
     }
     mark();
     const int nrep = (int)s->reps.size();
@@ -684,18 +670,13 @@ void enqueue_step(tdpd_sys *s, int p, cudaStream_t st, cudaEvent_t *ev = nullptr
         mark();
     }
     if (s->n_rbc && ev) {
-        const MemArgs m = mem_args(s, 1 - p, 1);
-        launch_mem_gather(m, st, true);
-        mark();
-        launch_mem_forces(m, st);
+        launch_membrane(mem_args(s, 1 - p, 1), st, true);
         mark();
     }
     const PairArgs pa = pair_args(s, nxt, 1, s->tile_sum[1 - p], s->disp[1 - p],
                                   pair_builds_lists(s) ? s->rb : nullptr);
     auto join = [&]() {
-        if (!branch) return;
-        cudaStreamWaitEvent(st, s->join, 0);
-        if (s->all_lagged) cudaStreamWaitEvent(st, s->gathered, 0);
+        if (branch) cudaStreamWaitEvent(st, s->join, 0);
     };
     if (!s->half) join();
     launch_pair(pa, st, PAIR_WALK);
@@ -793,9 +774,7 @@ void enqueue_init(tdpd_sys *s, cudaStream_t st, bool branch)
     if (branch) {
         cudaEventRecord(s->fork, st);
         cudaStreamWaitEvent(s->side, s->fork, 0);
-        const MemArgs m = mem_args(s, 1, 0);
-        launch_mem_gather(m, s->side, false);
-        launch_mem_forces(m, s->side);
+        launch_membrane(mem_args(s, 1, 0), s->side, false);
         cudaEventRecord(s->join, s->side);
     }
     launch_bin_init(s->buf[0], s->d_reps, N, s->count, s->tile_sum[0], s->cellrank, st);
@@ -812,11 +791,7 @@ void enqueue_init(tdpd_sys *s, cudaStream_t st, bool branch)
         launch_rank_gather(s->buf[0], s->buf[1], s->d_reps, s->keys, s->cellrank, s->cell_start, s->inv, N, ns, 0,
                            st, nullptr, 0, nullptr, 0, quarantine(s));
     }
-    if (s->n_rbc && !branch) {
-        const MemArgs m = mem_args(s, 1, 0);
-        launch_mem_gather(m, st, true);
-        launch_mem_forces(m, st);
-    }
+    if (s->n_rbc && !branch) launch_membrane(mem_args(s, 1, 0), st, true);
     const PairArgs pa = pair_args(s, s->buf[1], 0, s->tile_sum[1], s->disp[1],
                                   s->use_list && pair_builds_lists(s) ? s->rb_all : nullptr);
     if (branch && !s->half) cudaStreamWaitEvent(st, s->join, 0);
@@ -1375,9 +1350,6 @@ tdpd_status commit(tdpd_sys *s)
     s->lpp = striped_lists(s) ? 8 : 1;
     while (s->lpp < 8 && (long)N * s->lpp < 300000) s->lpp *= 2;
     s->n_rbc = (int)s->h_rbcs.size();
-    s->all_lagged = s->n_rbc > 0;
-    for (const HostRep &R : s->reps)
-        if (!R.rbcs.empty() && !R.mem.lagged_av) s->all_lagged = false;
     s->max_nv = max_nv;
     if (N == 0) return fail(s, TDPD_ESTATE, "no particles loaded");
 
@@ -1413,6 +1385,8 @@ tdpd_status commit(tdpd_sys *s)
         // largest degree) with each entry's cyclic neighbours
         std::vector<int> tri, t_tri(s->topos.size()), t_fan(s->topos.size()), t_stride(s->topos.size());
         std::vector<FanEntry> fan;
+        std::vector<int4> edge;
+        std::vector<int> t_edge(s->topos.size());
         for (size_t t = 0; t < s->topos.size(); ++t) {
             const Topo &T = s->topos[t];
             int mx = 0;
@@ -1420,6 +1394,17 @@ tdpd_status commit(tdpd_sys *s)
             t_tri[t] = (int)tri.size();
             t_fan[t] = (int)fan.size();
             t_stride[t] = mx;
+            // edge e = (a, b), a < b, with the third vertices of its two
+            // triangles: c where the triangle holds a -> b, d where b -> a
+            t_edge[t] = (int)edge.size();
+            for (const auto &e : T.edges) edge.push_back(make_int4(e.first, e.second, -1, -1));
+            int4 *te = edge.data() + t_edge[t];
+            for (int k = 0; k < T.ntri; ++k)
+                for (int q = 0; q < 3; ++q) {
+                    const int a = T.tri[3 * k + q], b = T.tri[3 * k + (q + 1) % 3], o = T.tri[3 * k + (q + 2) % 3];
+                    int4 &E = te[T.edge_id.at(std::make_pair(std::min(a, b), std::max(a, b)))];
+                    (a < b ? E.z : E.w) = o;
+                }
             tri.insert(tri.end(), T.tri.begin(), T.tri.end());
             for (int v = 0; v < T.nv; ++v) {
                 const int o = T.ring_off[v], deg = T.ring_off[v + 1] - o;
@@ -1427,8 +1412,11 @@ tdpd_status commit(tdpd_sys *s)
                     FanEntry F{-1, -1, -1, -1, -1, -1, 0, 0};
                     if (l < deg) {
                         const RingEntry &E = T.ring[o + l];
-                        F = FanEntry{E.nb, E.edge, E.tri, E.across, T.ring[o + (l + 1) % deg].nb,
-                                     T.ring[o + (l + deg - 1) % deg].nb, 0, 0};
+                        // the fan's triangle (v, nb, next) holds nb -> next
+                        const int next = T.ring[o + (l + 1) % deg].nb;
+                        const int far = T.edge_id.at(std::make_pair(std::min(E.nb, next), std::max(E.nb, next)));
+                        F = FanEntry{E.nb, E.edge, E.tri, E.across, next, T.ring[o + (l + deg - 1) % deg].nb,
+                                     E.edge | (v < E.nb ? 0 : 1) << 29, far | (E.nb < next ? 2 : 3) << 29};
                     }
                     fan.push_back(F);
                 }
@@ -1437,17 +1425,18 @@ tdpd_status commit(tdpd_sys *s)
         for (RbcDev &D : s->h_rbcs) {
             D.tri_off = t_tri[D.topo];
             D.fan_off = t_fan[D.topo];
+            D.edge_off = t_edge[D.topo];
             D.fan_stride = t_stride[D.topo];
         }
         if ((rc = dalloc(s, &s->d_rbcs, s->n_rbc)) || (rc = dalloc(s, &s->d_tri, tri.size())) ||
-            (rc = dalloc(s, &s->d_fan, fan.size())) || (rc = dalloc(s, &s->d_a0j, a0j.size())) ||
+            (rc = dalloc(s, &s->d_fan, fan.size())) || (rc = dalloc(s, &s->d_edge, edge.size())) || (rc = dalloc(s, &s->d_a0j, a0j.size())) ||
             (rc = dalloc(s, &s->d_bond, bond.size())) || (rc = dalloc(s, &s->d_ref[0], s->n_rbc)) ||
             (rc = dalloc(s, &s->d_ref[1], s->n_rbc)) || (rc = dalloc(s, &s->d_av[0], s->n_rbc)) ||
             (rc = dalloc(s, &s->d_av[1], s->n_rbc)) || (rc = dalloc(s, &s->d_cgv[0], s->n_rbc)) ||
             (rc = dalloc(s, &s->d_cgv[1], s->n_rbc)))
             return rc;
         if ((rc = upload(s, s->d_rbcs, s->h_rbcs.data(), s->n_rbc)) || (rc = upload(s, s->d_tri, tri.data(), tri.size())) ||
-            (rc = upload(s, s->d_fan, fan.data(), fan.size())) || (rc = upload(s, s->d_a0j, a0j.data(), a0j.size())) ||
+            (rc = upload(s, s->d_fan, fan.data(), fan.size())) || (rc = upload(s, s->d_edge, edge.data(), edge.size())) || (rc = upload(s, s->d_a0j, a0j.data(), a0j.size())) ||
             (rc = upload(s, s->d_bond, bond.data(), bond.size())))
             return rc;
     }
@@ -1506,7 +1495,6 @@ tdpd_status commit(tdpd_sys *s)
     CU(cudaStreamCreateWithFlags(&s->side, cudaStreamNonBlocking));
     CU(cudaEventCreateWithFlags(&s->fork, cudaEventDisableTiming));
     CU(cudaEventCreateWithFlags(&s->join, cudaEventDisableTiming));
-    CU(cudaEventCreateWithFlags(&s->gathered, cudaEventDisableTiming));
     if (!shapes.empty() && (rc = tune_shape(s, shapes))) return rc;
     if (s->lanes_fixed == 0 && (rc = autotune(s))) return rc;
     if ((rc = tune_sort(s))) return rc;
@@ -1989,6 +1977,7 @@ tdpd_status config_hash(tdpd_sys *s, uint64_t *out)
     if (s->n_rbc) {
         std::vector<RbcDev> R(s->n_rbc);
         CU(cudaMemcpy(R.data(), s->d_rbcs, sizeof(RbcDev) * R.size(), cudaMemcpyDeviceToHost));
+        for (RbcDev &D : R) D.edge_off = 0;       // (a derived table's offset, not part of the hash)
         h = fnv1a(R.data(), sizeof(RbcDev) * R.size(), h);
     }
     *out = h;

@@ -1,27 +1,28 @@
-// Membrane forces of the triangulated RBC model (Sec. 2.2, Eq. 10-16).
+// Membrane forces of the triangulated RBC model (Sec. 2.2, Eq. 10-16), one CTA per
+// membrane (k_membrane):
+//   - K-Gather of Sec. 3.3: the triangle areas and signed tetrahedron volumes and
+//     the vertex centroid (the next step's reference point), binary32 terms in
+//     compensated float-float sums, converted to binary64 once, and the
+//     constraint coefficients they give;
+//   - every edge once: the bond (WLC + POW, viscous and random parts) and the
+//     dihedral of its two triangles, their forces on the edge's four vertices
+//     left in shared memory;
+//   - K-Apply: every vertex sums, over its one-ring fan, the forces of its bonds
+//     and dihedrals and the area and volume gradients of its triangles. No
+//     atomics, a fixed order. A lagged membrane uses the previous step's
+//     coefficients, the others wait for this step's.
 //
-// k_mem_gather (K-Gather of Sec. 3.3): one CTA per membrane sums the
-//   triangle areas and signed tetrahedron volumes in FP64 with compensation,
-//   the constraint coefficients they give, and the vertex centroid that
-//   becomes the next step's reference point. A lagged membrane's K-Apply
-//   uses the previous step's coefficients, so it need not wait for this.
-// k_mem_forces (K-Apply, bonds and bending): eight lanes per vertex; lane l
-//   takes the l-th entry of the vertex's one-ring fan and adds
-//     - the bond (v, nb[l]): WLC + POW, viscous and random parts,
-//     - the dihedral on edge (v, nb[l]) (v as an edge end),
-//     - the triangle (v, nb[l], nb[l+1]): area and volume constraints,
-//     - the dihedral on edge (nb[l], nb[l+1]) (v as the opposite vertex);
-//   a shuffle sums the lanes. Every vertex force is written once, no atomics.
-//
-// Both kernels read the vertices' predicted positions and v~ from arrays in
-// load order (written by the previous step's pair kernel, or by the packing of
-// a loaded state) and write the force in load order, so they do not
-// depend on the cell sort and run beside it.
+// The vertices' predicted positions and v~ come from arrays in load order (written
+// by the previous step's pair kernel, or by the packing of a loaded state) and the
+// force goes out in load order, so the kernel does not depend on the cell sort and
+// runs beside it.
 //
 // Coordinates are taken relative to a per-membrane reference point with the
 // minimum image, so a membrane may straddle the periodic boundary as long as
-// it spans less than half a box. K-Gather's vertex centroid is the next
-// step's reference point; a loaded state's comes from k_mem_ref.
+// it spans less than half a box. The vertex centroid is the next step's reference
+// point; a loaded state's comes from k_mem_ref.
+#include <cooperative_groups.h>
+
 #include "launch.h"
 
 namespace tdpd {
@@ -43,181 +44,104 @@ __device__ __forceinline__ float3 rel_pos(const RepParams &P, float4 x, float4 r
                        min_image(x.z - ref.z, P.L[2], P.periodic[2]));
 }
 
-// Vertices of a membrane staged in shared memory by K-Gather (larger
-// membranes read their triangle corners from global memory).
-constexpr int GATHER_STAGE_NV = 2048;
-constexpr int GATHER_THREADS = 512;
+constexpr int MEM_THREADS = 512;
 constexpr int REF_THREADS = 256;
 
-// K-Gather: one CTA of GATHER_THREADS per membrane (512 at 64 registers: two
-// CTAs per SM, twice the resident membranes of 1024-thread CTAs; 46 -> 28 us
-// on the 512-replica ensemble); each thread takes two triangles and one
-// vertex of a 500-vertex cell (prefetched together); the
-// binary32 terms are reduced with compensated float-float sums (warp
-// shuffles, then one warp over the warp totals) and converted to binary64 once.
-// The triangle indices and the vertex positions are loaded together (the
-// positions, relative to the reference point, into shared memory), so a cold
-// start costs two dependent memory round trips, not three.
-__global__ void __launch_bounds__(GATHER_THREADS, 2) k_mem_gather(MemArgs A)
+// Dynamic shared memory of one of the C CTAs of a membrane: every vertex's
+// position and velocity, and for its share of the edges the force on each edge's
+// four vertices (three planes of 4 x the share), of the triangles their area and
+// volume.
+__host__ __device__ constexpr int share_of(int n, int C) { return (n + C - 1) / C; }
+static size_t membrane_smem(int nv, int C)
 {
+    return (size_t)nv * 32 + (size_t)share_of(3 * nv - 6, C) * 48 + (size_t)share_of(2 * nv - 4, C) * 8;
+}
+
+// C CTAs (a thread-block cluster; CL false: one CTA) per membrane. Each stages all
+// its vertices, computes a share of the edges and triangles and sums a share of
+// the vertices, reading the other shares through distributed shared memory. Every
+// sum has an order of its own, whatever C is (a triangle's terms are added by
+// thread t mod 512, a vertex's fan by eight lanes), so a membrane gives the same
+// bits alone and in a batch.
+//
+// Bound by the arithmetic, above all the five TEA draws and ten normals of a
+// bond's random force (about 650 of 900 instructions per edge). Computed from each
+// of its ends, with the dihedral from each of its four vertices (eight lanes per
+// vertex over its fan), this took 47 us on the 229 cells of 128 replicas after a
+// K-Gather of 8 us; every edge once: 38 us in one launch. A single cell is a chain of
+// latencies: 22 us in one CTA, 12.4 in four (12.0 in the two kernels before).
+template <bool CL>
+__global__ void __launch_bounds__(MEM_THREADS, 2) k_membrane(MemArgs A)
+{
+    namespace cg = cooperative_groups;
     pdl_enter();
-    const int b = blockIdx.x;
-    if (b == 0 && threadIdx.x == 0) A.mem_ctr[1 - A.q] = A.mem_ctr[A.q] + 1u;   // the next evaluation's
+    extern __shared__ float4 mem_sm[];
+    __shared__ FF sh[MEM_THREADS / 32][5];
+    __shared__ float2 cgv_sh;
+    cg::cluster_group cl = cg::this_cluster();
+    const int C = CL ? (int)cl.num_blocks() : 1, rank = CL ? (int)cl.block_rank() : 0;
+    const int b = blockIdx.x / C, tid = threadIdx.x;
+    if (blockIdx.x == 0 && tid == 0) A.mem_ctr[1 - A.q] = A.mem_ctr[A.q] + 1u;   // the next evaluation's
     const RbcDev R = A.rbcs[b];
     const RepParams &P = A.reps[R.rep];
     const float4 ref = A.ref_in[b];
+    const int es = share_of(R.ne, C), ts = share_of(R.ntri, C);
+    float4 *xs = mem_sm, *vs = xs + R.nv;
+    float *fx = reinterpret_cast<float *>(vs + R.nv);        // fy, fz: the next planes of 4 es
+    float2 *tri_av = reinterpret_cast<float2 *>(fx + 12 * es);
     const int *tri = A.tri + R.tri_off;
-    __shared__ float4 xs[GATHER_STAGE_NV];
-    const bool staged = R.nv <= GATHER_STAGE_NV;
-    int3 pre[2];
-#pragma unroll
-    for (int u = 0; u < 2; ++u) {
-        const int t = threadIdx.x + u * blockDim.x;
-        pre[u] = t < R.ntri ? make_int3(tri[3 * t], tri[3 * t + 1], tri[3 * t + 2]) : make_int3(0, 0, 0);
-    }
+
+    // vertices, and this CTA's first triangle and edge in flight with them
+    const int t0 = rank * ts, t1 = min(t0 + ts, R.ntri), e0 = rank * es, e1 = min(e0 + es, R.ne);
+    const int tp = t0 + tid, ep = e0 + tid;
+    int3 tv = tp < t1 ? make_int3(tri[3 * tp], tri[3 * tp + 1], tri[3 * tp + 2]) : make_int3(0, 0, 0);
+    int4 E = ep < e1 ? A.edge[R.edge_off + ep] : make_int4(0, 0, 0, 0);
     FF v[5];
 #pragma unroll
     for (int k = 0; k < 5; ++k) v[k] = FF{0.0f, 0.0f};
-    for (int k = threadIdx.x; k < R.nv; k += blockDim.x) {
+    for (int k = tid; k < R.nv; k += MEM_THREADS) {
         const float3 x = rel_pos(P, A.mx[R.gbase + k], ref);
-        if (staged) xs[k] = make_float4(x.x, x.y, x.z, 0.0f);
+        xs[k] = make_float4(x.x, x.y, x.z, 0.0f);
+        vs[k] = A.mv[R.gbase + k];
         v[2] = ff_add(v[2], x.x);
         v[3] = ff_add(v[3], x.y);
         v[4] = ff_add(v[4], x.z);
     }
     __syncthreads();
-    int u = 0;
-    for (int t = threadIdx.x; t < R.ntri; t += blockDim.x, ++u) {
-        const int3 tv = u == 0 ? pre[0] : u == 1 ? pre[1] : make_int3(tri[3 * t], tri[3 * t + 1], tri[3 * t + 2]);
-        float3 x0, x1, x2;
-        if (staged) {
-            x0 = f3(xs[tv.x]);
-            x1 = f3(xs[tv.y]);
-            x2 = f3(xs[tv.z]);
-        } else {
-            x0 = rel_pos(P, A.mx[R.gbase + tv.x], ref);
-            x1 = rel_pos(P, A.mx[R.gbase + tv.y], ref);
-            x2 = rel_pos(P, A.mx[R.gbase + tv.z], ref);
-        }
+    for (int t = tp; t < t1; t += MEM_THREADS) {
+        if (t != tp) tv = make_int3(tri[3 * t], tri[3 * t + 1], tri[3 * t + 2]);
+        const float3 x0 = f3(xs[tv.x]), x1 = f3(xs[tv.y]), x2 = f3(xs[tv.z]);
         const float3 n = cross(sub(x1, x0), sub(x2, x0));
-        v[0] = ff_add(v[0], 0.5f * sqrtf(dot(n, n)));
-        v[1] = ff_add(v[1], dot(x0, cross(x1, x2)) * (1.0f / 6.0f));
+        tri_av[t - t0] = make_float2(0.5f * sqrtf(dot(n, n)), dot(x0, cross(x1, x2)) * (1.0f / 6.0f));
     }
-    __shared__ FF sh[32][5];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-        for (int k = 0; k < 5; ++k) v[k] = ff_add(v[k], ff_shfl_down(v[k], o));
-    if (lane == 0)
-        for (int k = 0; k < 5; ++k) sh[w][k] = v[k];
-    __syncthreads();
-    if (w != 0) return;
-#pragma unroll
-    for (int k = 0; k < 5; ++k) v[k] = lane < nw ? sh[lane][k] : FF{0.0f, 0.0f};
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-        for (int k = 0; k < 5; ++k) v[k] = ff_add(v[k], ff_shfl_down(v[k], o));
-    if (lane == 0) {
-        const double Ab = ff_value(v[0]), Vb = ff_value(v[1]);
-        A.av_out[b] = make_double2(Ab, Vb);
-        // constraint coefficients of Eq. 14-15, once per membrane in binary64
-        // (divisions by A0, V0 and nv were done once on the host)
-        A.cgv_out[b] = make_float2((float)((Ab - R.A0) * R.kgA0), (float)((Vb - R.V0) * R.kvV0));
-        const double inv = R.inv_nv;
-        float c3[3] = {(float)(ref.x + ff_value(v[2]) * inv), (float)(ref.y + ff_value(v[3]) * inv),
-                       (float)(ref.z + ff_value(v[4]) * inv)};
-        for (int c = 0; c < 3; ++c)
-            if (P.periodic[c]) {
-                if (c3[c] < 0.0f) c3[c] += P.L[c];
-                else if (c3[c] >= P.L[c]) c3[c] -= P.L[c];
-            }
-        A.ref_out[b] = make_float4(c3[0], c3[1], c3[2], 0.0f);
-    }
-}
-
-// Gradient of the angle theta between the outward normals of triangles
-// (a, b, c) and (b, a, d) (positive on a convex fold). Returns sin and cos of
-// theta; role selects the vertex whose gradient is written to g.
-struct Dihedral {
-    float sin_t, cos_t;
-    float3 g;
-};
-
-__device__ __forceinline__ Dihedral dihedral(float3 xa, float3 xb, float3 xc, float3 xd, int role)
-{
-    const float3 e = sub(xb, xa);
-    const float3 n1 = cross(e, sub(xc, xa));
-    const float3 n2 = cross(sub(xa, xb), sub(xd, xb));
-    const float le2 = dot(e, e), n1s = dot(n1, n1), n2s = dot(n2, n2);
-    const float le = sqrtf(le2);
-    const float inv12 = rsqrtf(n1s * n2s);
-    Dihedral D;
-    D.cos_t = dot(n1, n2) * inv12;
-    D.sin_t = dot(cross(n1, n2), e) * inv12 / le;
-    const float3 u1 = scl(1.0f / n1s, n1), u2 = scl(1.0f / n2s, n2);
-    if (role == 0) {          // a
-        const float p1 = dot(sub(xc, xb), e) / le, p2 = dot(sub(xd, xb), e) / le;
-        D.g = scl(-1.0f, add(scl(p1, u1), scl(p2, u2)));
-    } else {                  // c
-        D.g = scl(-le, u1);
-    }
-    return D;
-}
-
-// Four CTAs per SM (64 registers, a few spilled to L1): faster than two or
-// three on the ensemble of many membranes.
-__global__ void __launch_bounds__(256, 4) k_mem_forces(MemArgs A)
-{
-    pdl_enter();
-    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) A.mem_ctr[1 - A.q] = A.mem_ctr[A.q] + 1u;
-    const int b = blockIdx.y;
-    const RbcDev R = A.rbcs[b];
-    const int v = (blockIdx.x * blockDim.x + threadIdx.x) >> 3;
-    const int lane8 = threadIdx.x & 7;
-    const bool live = v < R.nv;
-    const RepParams &P = A.reps[R.rep];
-    float3 f = make_float3(0.f, 0.f, 0.f);
-    if (live) {
-        const float4 ref = A.ref_in[b];
-        const float2 cgv = P.m_lagged ? A.cgv_lag[b] : A.cgv_seq[b];
-        const float cg = cgv.x, cv = cgv.y;
-        const FanEntry *fan = A.fan + R.fan_off + (size_t)v * R.fan_stride;
-        const float3 xv = rel_pos(P, A.mx[R.gbase + v], ref);
-        const float4 vv = A.mv[R.gbase + v];
-        const uint32_t idv = (uint32_t)(R.gbase + v - P.pbase);
+    // edges (a, b), triangles (a, b, c) and (b, a, d)
+    {
         const uint32_t step = A.mem_ctr[A.q] + P.step0;
-        for (int l = lane8; l < R.fan_stride; l += 8) {
-            const FanEntry E = fan[l];
-            if (E.nb < 0) break;                      // past the vertex's degree
-            const float3 xl = rel_pos(P, A.mx[R.gbase + E.nb], ref);
-            const float3 xn = rel_pos(P, A.mx[R.gbase + E.nb_next], ref);
-            const float3 xp = rel_pos(P, A.mx[R.gbase + E.nb_prev], ref);
-            const float3 xw = rel_pos(P, A.mx[R.gbase + E.across], ref);
-
-            // bond (v, nb[l]): Eq. 10-13
+        const int id0 = R.gbase - P.pbase;
+        for (int e = ep; e < e1; e += MEM_THREADS) {
+            if (e != ep) E = A.edge[R.edge_off + e];
+            const float2 bp = A.bond[R.bond_off + e];        // (l_m, k_p)
+            const float3 xa = f3(xs[E.x]), xb = f3(xs[E.y]), xc = f3(xs[E.z]), xd = f3(xs[E.w]);
+            const float3 d = sub(xb, xa);
+            const float l2 = dot(d, d);
+            // bond, the force on a: Eq. 10-13 (ue points from b to a)
+            float3 f;
             {
-                const float3 d = sub(xv, xl);
-                const float l2 = dot(d, d);
                 const float il = rsqrtf(l2);
                 const float len = l2 * il;
-                const float3 e = scl(il, d);
-                const float2 bp = A.bond[R.bond_off + E.edge];   // (l_m, k_p)
+                const float3 ue = scl(-il, d);
                 const float x = len / bp.x;
                 const float omx = 1.0f - x;
                 const float pw = P.m_m == 2.0f ? len * len : __powf(len, P.m_m);
                 const float dudl = P.m_wlc0 * (0.25f / (omx * omx) - 0.25f + x) - bp.y / pw;
-                f = add(f, scl(-dudl, e));
-                const float4 vl = A.mv[R.gbase + E.nb];
-                const float3 vij = make_float3(vv.x - vl.x, vv.y - vl.y, vv.z - vl.z);
-                const float ve = dot(vij, e);
-                f = add(f, add(scl(-P.m_gT, vij), scl(-P.m_gC * ve, e)));
-                const uint32_t idl = (uint32_t)(R.gbase + E.nb - P.pbase);
+                const float3 vij = sub(f3(vs[E.x]), f3(vs[E.y]));
+                const float ve = dot(vij, ue);
+                f = add(scl(-dudl, ue), add(scl(-P.m_gT, vij), scl(-P.m_gC * ve, ue)));
                 float z[10];
 #pragma unroll
                 for (int s = 0; s < 5; ++s) {
-                    const float2 g = normal2(pair_bits(idv, idl, P.seed_lo, P.seed_hi, step, 1u + s));
+                    const float2 g = normal2(pair_bits((uint32_t)(id0 + E.x), (uint32_t)(id0 + E.y), P.seed_lo,
+                                                       P.seed_hi, step, 1u + s));
                     z[2 * s] = g.x;
                     z[2 * s + 1] = g.y;
                 }
@@ -225,43 +149,133 @@ __global__ void __launch_bounds__(256, 4) k_mem_forces(MemArgs A)
                 // (W^S - tr/3 I) e with W^S the symmetric part of Z
                 const float s01 = 0.5f * (z[1] + z[3]), s02 = 0.5f * (z[2] + z[6]), s12 = 0.5f * (z[5] + z[7]);
                 const float t3 = tr * (1.0f / 3.0f);
-                const float3 we = make_float3((z[0] - t3) * e.x + s01 * e.y + s02 * e.z,
-                                              s01 * e.x + (z[4] - t3) * e.y + s12 * e.z,
-                                              s02 * e.x + s12 * e.y + (z[8] - t3) * e.z);
-                f = add(f, add(scl(P.m_rand_T, we), scl(P.m_rand_C * tr, e)));
+                const float3 we = make_float3((z[0] - t3) * ue.x + s01 * ue.y + s02 * ue.z,
+                                              s01 * ue.x + (z[4] - t3) * ue.y + s12 * ue.z,
+                                              s02 * ue.x + s12 * ue.y + (z[8] - t3) * ue.z);
+                f = add(f, add(scl(P.m_rand_T, we), scl(P.m_rand_C * tr, ue)));
             }
-            // dihedral on edge (v, nb[l]): triangles (v, nb[l], nb[l+1]), (nb[l], v, nb[l-1])
-            {
-                const Dihedral D = dihedral(xv, xl, xn, xp, 0);
-                const float s = P.m_kb * (D.sin_t * P.m_cos0 - D.cos_t * P.m_sin0);
-                f = sub(f, scl(s, D.g));
-            }
-            // triangle (v, nb[l], nb[l+1]): Eq. 14-15
-            {
-                const float3 n = cross(sub(xl, xv), sub(xn, xv));
-                const float nn = sqrtf(dot(n, n));
-                const float At = 0.5f * nn;
-                const float a0 = A.a0j[R.a0j_off + E.tri];
-                const float ca = cg + P.m_kl * (At - a0) / a0;
-                const float3 gA = scl(0.5f / nn, cross(n, sub(xn, xl)));
-                const float3 gV = scl(1.0f / 6.0f, cross(xl, xn));
-                f = sub(f, add(scl(ca, gA), scl(cv, gV)));
-            }
-            // dihedral on edge (nb[l], nb[l+1]) with v opposite: (nb[l], nb[l+1], v), (nb[l+1], nb[l], w)
-            {
-                const Dihedral D = dihedral(xl, xn, xv, xw, 2);
-                const float s = P.m_kb * (D.sin_t * P.m_cos0 - D.cos_t * P.m_sin0);
-                f = sub(f, scl(s, D.g));
+            // dihedral: the gradients of the angle theta between the outward
+            // normals (positive on a convex fold) times -kb sin(theta - theta0)
+            const float3 n1 = cross(d, sub(xc, xa));
+            const float3 n2 = cross(sub(xd, xb), d);
+            const float n1s = dot(n1, n1), n2s = dot(n2, n2);
+            const float le = sqrtf(l2), inv12 = rsqrtf(n1s * n2s);
+            const float cos_t = dot(n1, n2) * inv12;
+            const float sin_t = dot(cross(n1, n2), d) * inv12 / le;
+            const float s = P.m_kb * (sin_t * P.m_cos0 - cos_t * P.m_sin0);
+            const float3 u1 = scl(1.0f / n1s, n1), u2 = scl(1.0f / n2s, n2);
+            const float a1 = dot(sub(xc, xb), d) / le, a2 = dot(sub(xd, xb), d) / le;
+            const float b1 = dot(sub(xa, xc), d) / le, b2 = dot(sub(xa, xd), d) / le;
+            const float3 fo[4] = {add(f, scl(s, add(scl(a1, u1), scl(a2, u2)))),
+                                  sub(scl(s, add(scl(b1, u1), scl(b2, u2))), f), scl(s * le, u1), scl(s * le, u2)};
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                float *o = fx + k * es + (e - e0);
+                o[0] = fo[k].x;
+                o[4 * es] = fo[k].y;
+                o[8 * es] = fo[k].z;
             }
         }
     }
-#pragma unroll
-    for (int o = 4; o > 0; o >>= 1) {
-        f.x += __shfl_xor_sync(0xffffffffu, f.x, o);
-        f.y += __shfl_xor_sync(0xffffffffu, f.y, o);
-        f.z += __shfl_xor_sync(0xffffffffu, f.z, o);
+    if (CL) cl.sync();
+    else __syncthreads();
+
+    // the totals, by every CTA of the membrane
+    const int lane = tid & 31, w = tid >> 5;
+    for (int t = tid; t < R.ntri; t += MEM_THREADS) {
+        float2 av;
+        if (CL) {
+            const int r = t / ts;
+            av = cl.map_shared_rank(tri_av, r)[t - r * ts];
+        } else {
+            av = tri_av[t];
+        }
+        v[0] = ff_add(v[0], av.x);
+        v[1] = ff_add(v[1], av.y);
     }
-    if (live && lane8 == 0) A.fext[R.gbase + v] = make_float4(f.x, f.y, f.z, 0.0f);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int k = 0; k < 5; ++k) v[k] = ff_add(v[k], ff_shfl_down(v[k], o));
+    if (lane == 0)
+        for (int k = 0; k < 5; ++k) sh[w][k] = v[k];
+    __syncthreads();
+    if (w == 0) {
+        constexpr int NW = MEM_THREADS / 32;
+#pragma unroll
+        for (int k = 0; k < 5; ++k) v[k] = lane < NW ? sh[lane][k] : FF{0.0f, 0.0f};
+#pragma unroll
+        for (int o = NW / 2; o > 0; o >>= 1)
+#pragma unroll
+            for (int k = 0; k < 5; ++k) v[k] = ff_add(v[k], ff_shfl_down(v[k], o));
+        if (lane == 0) {
+            const double Ab = ff_value(v[0]), Vb = ff_value(v[1]);
+            // constraint coefficients of Eq. 14-15, once per membrane in binary64
+            // (divisions by A0, V0 and nv were done once on the host)
+            const float2 cgv = make_float2((float)((Ab - R.A0) * R.kgA0), (float)((Vb - R.V0) * R.kvV0));
+            cgv_sh = P.m_lagged && A.cgv_lag ? A.cgv_lag[b] : cgv;
+            if (rank == 0) {
+                A.av_out[b] = make_double2(Ab, Vb);
+                A.cgv_out[b] = cgv;
+                const double inv = R.inv_nv;
+                float c3[3] = {(float)(ref.x + ff_value(v[2]) * inv), (float)(ref.y + ff_value(v[3]) * inv),
+                               (float)(ref.z + ff_value(v[4]) * inv)};
+                for (int c = 0; c < 3; ++c)
+                    if (P.periodic[c]) {
+                        if (c3[c] < 0.0f) c3[c] += P.L[c];
+                        else if (c3[c] >= P.L[c]) c3[c] -= P.L[c];
+                    }
+                A.ref_out[b] = make_float4(c3[0], c3[1], c3[2], 0.0f);
+            }
+        }
+    }
+    __syncthreads();
+
+    // a share of the vertices, eight lanes each over the fan
+    const float c_area = cgv_sh.x, c_vol = cgv_sh.y;
+    const int vsh = share_of(R.nv, C), v0 = rank * vsh, v1 = min(v0 + vsh, R.nv);
+    auto edge_force = [&](int code) {
+        const int role = code >> 29, e = code & ((1 << 29) - 1);
+        const float *o;
+        if (CL) {
+            const int r = e / es;
+            o = cl.map_shared_rank(fx, r) + role * es + (e - r * es);
+        } else {
+            o = fx + role * es + e;
+        }
+        return make_float3(o[0], o[4 * es], o[8 * es]);
+    };
+    for (int k0 = v0; k0 < v1; k0 += MEM_THREADS / 8) {
+        const int k = k0 + (tid >> 3);
+        float3 f = make_float3(0.f, 0.f, 0.f);
+        if (k < v1) {
+            const FanEntry *fan = A.fan + R.fan_off + (size_t)k * R.fan_stride;
+            const float3 xv = f3(xs[k]);
+            for (int l = tid & 7; l < R.fan_stride; l += 8) {
+                const FanEntry F = fan[l];
+                if (F.nb < 0) break;                      // past the vertex's degree
+                f = add(f, add(edge_force(F.end), edge_force(F.opp)));
+                // triangle (v, nb[l], nb[l+1]): Eq. 14-15
+                const float3 xl = f3(xs[F.nb]), xn = f3(xs[F.nb_next]);
+                const float3 n = cross(sub(xl, xv), sub(xn, xv));
+                const float nn = sqrtf(dot(n, n));
+                const float At = 0.5f * nn;
+                const float a0 = A.a0j[R.a0j_off + F.tri];
+                const float ca = c_area + P.m_kl * (At - a0) / a0;
+                const float3 gA = scl(0.5f / nn, cross(n, sub(xn, xl)));
+                const float3 gV = scl(1.0f / 6.0f, cross(xl, xn));
+                f = sub(f, add(scl(ca, gA), scl(c_vol, gV)));
+            }
+        }
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) {
+            f.x += __shfl_xor_sync(0xffffffffu, f.x, o);
+            f.y += __shfl_xor_sync(0xffffffffu, f.y, o);
+            f.z += __shfl_xor_sync(0xffffffffu, f.z, o);
+        }
+        if (k < v1 && (tid & 7) == 0) A.fext[R.gbase + k] = make_float4(f.x, f.y, f.z, 0.0f);
+    }
+    if (CL) cl.sync();                 // the shares stay until every CTA has read them
 }
 
 // Reference point of each membrane of a loaded state, from the uploaded
@@ -370,18 +384,37 @@ void launch_mem_ref(const float *x3, const RbcDev *rbcs, const FanEntry *fan, co
     }
 }
 
-void launch_mem_gather(const MemArgs &a, cudaStream_t st, bool pdl)
-{
-    if (a.n_rbc <= 0) return;
-    if (pdl) launch_pdl(k_mem_gather, a.n_rbc, GATHER_THREADS, st, a);
-    else k_mem_gather<<<a.n_rbc, GATHER_THREADS, 0, st>>>(a);
-}
+// CTAs per membrane: the most (of 1, 2, 4) that leave one to two CTAs per SM
+static int membrane_ctas(int n_rbc) { return n_rbc <= 76 ? 4 : n_rbc <= 152 ? 2 : 1; }
 
-void launch_mem_forces(const MemArgs &a, cudaStream_t st)
+void launch_membrane(const MemArgs &a, cudaStream_t st, bool pdl)
 {
     if (a.n_rbc <= 0) return;
-    dim3 g((a.max_nv * 8 + 255) / 256, a.n_rbc);
-    launch_pdl(k_mem_forces, g, 256, st, a);
+    const int C = membrane_ctas(a.n_rbc);
+    auto kern = C > 1 ? k_membrane<true> : k_membrane<false>;
+    const size_t smem = membrane_smem(a.max_nv, C);
+    if (smem > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = a.n_rbc * C;
+    cfg.blockDim = MEM_THREADS;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[2];
+    int n = 0;
+    if (C > 1) {
+        at[n].id = cudaLaunchAttributeClusterDimension;
+        at[n].val.clusterDim.x = C;
+        at[n].val.clusterDim.y = at[n].val.clusterDim.z = 1;
+        ++n;
+    }
+    if (pdl) {
+        at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[n].val.programmaticStreamSerializationAllowed = 1;
+        ++n;
+    }
+    cfg.attrs = at;
+    cfg.numAttrs = n;
+    cudaLaunchKernelEx(&cfg, kern, a);
 }
 
 }  // namespace tdpd

@@ -112,14 +112,14 @@ struct MemArgs {
     const RbcDev *rbcs;
     const int *tri;              // triangle table (RbcDev::tri_off)
     const FanEntry *fan;         // fan table (RbcDev::fan_off, fan_stride)
+    const int4 *edge;            // edge table (RbcDev::edge_off): a, b, c, d with triangles (a, b, c), (b, a, d)
     const float *a0j;
     const float2 *bond;          // (l_m, k_p) per bond
     const float4 *ref_in;        // per-membrane reference point
     float4 *ref_out;             // next reference point (centroid)
     double2 *av_out;             // per-membrane (A, V) of these positions
     float2 *cgv_out;             // their constraint coefficients k_g (A - A0)/A0, k_v (V - V0)/V0
-    const float2 *cgv_seq;       // coefficients K-Apply uses (this step's) ...
-    const float2 *cgv_lag;       // ... or the previous step's, for a lagged replica
+    const float2 *cgv_lag;       // the coefficients K-Apply uses for a lagged replica (the previous step's; null: this one's)
     float4 *fext;                // membrane force by load index
     uint32_t *mem_ctr;           // [2] step counters of the membrane kernels: this
     int q;                       // evaluation reads mem_ctr[q], sets mem_ctr[1-q] to it + 1
@@ -223,8 +223,7 @@ void launch_list_build(const ListArgs &a, cudaStream_t st);
 void launch_mem_ref(const float *x3, const RbcDev *rbcs, const FanEntry *fan, const RepParams *reps, float4 *ref_out,
                     int n_rbc, int max_nv, int max_stride, cudaStream_t st);
 // pdl: launched as a programmatic dependent of the previous kernel on st
-void launch_mem_gather(const MemArgs &a, cudaStream_t st, bool pdl);
-void launch_mem_forces(const MemArgs &a, cudaStream_t st);
+void launch_membrane(const MemArgs &a, cudaStream_t st, bool pdl);
 // chunks: (replica, first slot, end slot); part: OBS_K doubles per chunk;
 // total: their sums over the chunks in chunk order (binary64); done: a
 // counter at zero, left at zero
