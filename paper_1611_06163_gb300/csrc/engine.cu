@@ -582,6 +582,10 @@ SortSmallArgs sort_small_args(tdpd_sys *s, int p)
     return a;
 }
 
+// Tiles the scan covers: those of the cells and of the end of the last one (the
+// arrays hold the largest candidate shape's).
+int scan_tiles(const tdpd_sys *s) { return std::min(s->n_tiles, s->NC / SCAN_TILE + 1); }
+
 // Cells the one-cluster sort may scan (its particle limit depends on the
 // cluster size: SORT_SMALL_ITEMS per thread).
 constexpr int SORT_SMALL_MAX_NC = 1 << 20;
@@ -638,16 +642,18 @@ void enqueue_step(tdpd_sys *s, int p, cudaStream_t st, cudaEvent_t *ev = nullptr
             mark();
         } else if (inline_decide(s)) {
             const DecideArgs d{s->disp[p], s->disp[1 - p], s->rb, s->step_ctr, s->builds, nrep};
-            launch_bin_next(cur, s->d_reps, s->N, s->count, s->tile_sum[0], s->cellrank, s->rb, any, st, d);
+            launch_bin_next(nxt.pos, cur.vel, s->d_reps, nrep, s->N, s->count, s->tile_sum[0], s->cellrank, s->rb, any,
+                            st, d);
             mark();
         } else {
             launch_rebuild_decide(s->disp[p], s->disp[1 - p], s->rb, s->d_reps, nrep, 0, s->step_ctr, s->builds, st);
             mark();
-            launch_bin_next(cur, s->d_reps, s->N, s->count, s->tile_sum[0], s->cellrank, s->rb, any, st);
+            launch_bin_next(nxt.pos, cur.vel, s->d_reps, nrep, s->N, s->count, s->tile_sum[0], s->cellrank, s->rb, any,
+                            st);
             mark();
         }
         if (!s->sort_ctas) {
-            launch_scan(s->count, s->cell_start, s->n_tiles, s->tile_sum[0], s->tile_sum[1], s->step_ctr, 0, st,
+            launch_scan(s->count, s->cell_start, scan_tiles(s), s->tile_sum[0], s->tile_sum[1], s->step_ctr, 0, st,
                         any);
             mark();
             launch_scatter_keys(cur, s->cellrank, s->cell_start, s->keys, s->N, st, any, s->rb);
@@ -661,7 +667,7 @@ void enqueue_step(tdpd_sys *s, int p, cudaStream_t st, cudaEvent_t *ev = nullptr
             mark();
         }
     } else {
-        launch_scan(s->count, s->cell_start, s->n_tiles, s->tile_sum[p], s->tile_sum[1 - p], s->step_ctr, 1, st);
+        launch_scan(s->count, s->cell_start, scan_tiles(s), s->tile_sum[p], s->tile_sum[1 - p], s->step_ctr, 1, st);
         mark();
         launch_scatter_keys(cur, s->cellrank, s->cell_start, s->keys, s->N, st);
         mark();
@@ -778,7 +784,7 @@ void enqueue_init(tdpd_sys *s, cudaStream_t st, bool branch)
         cudaEventRecord(s->join, s->side);
     }
     launch_bin_init(s->buf[0], s->d_reps, N, s->count, s->tile_sum[0], s->cellrank, st);
-    launch_scan(s->count, s->cell_start, s->n_tiles, s->tile_sum[0], s->tile_sum[1], s->step_ctr, 0, st);
+    launch_scan(s->count, s->cell_start, scan_tiles(s), s->tile_sum[0], s->tile_sum[1], s->step_ctr, 0, st);
     launch_scatter_keys(s->buf[0], s->cellrank, s->cell_start, s->keys, N, st);
     if (s->use_list) {
         launch_rank_gather(s->buf[0], s->buf[1], s->d_reps, s->keys, s->cellrank, s->cell_start, s->inv, N, ns, 0,

@@ -50,15 +50,24 @@ __global__ void k_rebuild_decide(const uint32_t *__restrict__ disp, uint32_t *di
 }
 
 // Cell and rank of the position each particle of a rebuilding replica will
-// have at the next force evaluation (the predictor of the gather), for the
-// sort of a rebuild step. A replica that keeps its list keeps its slots: its
-// particles are not binned, and its whole count goes to its first cell, so
-// that the scan still gives every replica its own slot range.
-// With D.disp set (few replicas) the rebuild decision is taken here instead
-// of in k_rebuild_decide: every CTA reads the replicas' maxima itself, and
+// have at the next force evaluation (the last pair epilogue wrote it, for every
+// slot, into the other buffer: next_pos), for the sort of a rebuild step. A replica
+// that keeps its list keeps its slots: its particles are not binned, and its whole
+// count goes to its first cell, so that the scan still gives every replica its own
+// slot range. With D.disp set (few replicas) the rebuild decision is taken here
+// instead of in k_rebuild_decide: every CTA reads the replicas' maxima itself, and
 // CTA 0 records the decision as k_rebuild_decide would; otherwise rb holds it.
-__global__ void k_bin_next(Buffers b, const RepParams *__restrict__ reps, int n, int *count, int *tile_sum,
-                           int2 *cellrank, const uint32_t *any, const uint32_t *__restrict__ rb, DecideArgs D)
+// Bound by the ranks' round trip to the L2; two particles per thread and turn keep
+// two in flight (786k particles: 21.6 us; one per thread, with the positions
+// predicted again from three more arrays: 28.7). A step without a rebuild launches
+// it too, so the grid is at most what the GPU holds at once.
+constexpr int BIN_THREADS = 256, BIN_GRID_MAX = 152 * 8;
+__global__ void __launch_bounds__(BIN_THREADS) k_bin_next(const float4 *__restrict__ next_pos,
+                                                          const float4 *__restrict__ vel,
+                                                          const RepParams *__restrict__ reps, int n_rep, int n,
+                                                          int *count, int *tile_sum, int2 *cellrank,
+                                                          const uint32_t *any, const uint32_t *__restrict__ rb,
+                                                          DecideArgs D)
 {
     pdl_enter();
     if (D.disp) {
@@ -81,30 +90,40 @@ __global__ void k_bin_next(Buffers b, const RepParams *__restrict__ reps, int n,
     } else if (!*any) {
         return;
     }
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    int c = -1;
-    if (k < n) {
-        const float4 v = b.vel[k];
-        const int r = wbits(v.w);
-        const RepParams &P = reps[r];
-        const bool rebuild = D.disp ? __uint_as_float(D.disp[r]) > P.half_skin2 : rb[r] != 0u;
-        if (rebuild) {
-            const float4 p = b.pos[k];
-            const int type = (int)((uint32_t)wbits(p.w) >> 24);
-            float3 rn = make_float3(p.x, p.y, p.z);
-            if (!((P.frozen_mask >> type) & 1u)) {
-                bool flip;
-                rn = predict_pos(P, p, v, b.frc[k], flip);
+    const int G = gridDim.x * BIN_THREADS, first = blockIdx.x * BIN_THREADS + threadIdx.x;
+    // (a turn's bound is the same for the lanes of a warp)
+    for (int k0 = first; k0 - (int)(threadIdx.x & 31) < n; k0 += 2 * G) {
+        int c[2], rank[2], r[2];
+        float4 p[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int k = k0 + u * G;
+            c[u] = -1;
+            if (k < n) {
+                r[u] = n_rep > 1 ? wbits(vel[k].w) : 0;
+                p[u] = next_pos[k];
             }
-            c = cell_of(P, rn.x, rn.y, rn.z);
-            const int rank = atomicAdd(count + c, 1);
-            cellrank[k] = make_int2(c, rank);
-        } else if (k == P.pbase) {
-            atomicAdd(count + P.cell_base, P.n);
-            atomicAdd(tile_sum + (P.cell_base >> SCAN_TILE_LOG2), P.n);
+        }
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int k = k0 + u * G;
+            if (k >= n) continue;
+            const RepParams &P = reps[r[u]];
+            const bool rebuild = D.disp ? __uint_as_float(D.disp[r[u]]) > P.half_skin2 : rb[r[u]] != 0u;
+            if (rebuild) {
+                c[u] = cell_of(P, p[u].x, p[u].y, p[u].z);
+                rank[u] = atomicAdd(count + c[u], 1);
+            } else if (k == P.pbase) {
+                atomicAdd(count + P.cell_base, P.n);
+                atomicAdd(tile_sum + (P.cell_base >> SCAN_TILE_LOG2), P.n);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            add_tile_count(tile_sum, c[u]);
+            if (c[u] >= 0) cellrank[k0 + u * G] = make_int2(c[u], rank[u]);
         }
     }
-    add_tile_count(tile_sum, c);
 }
 
 // One thread per pair lane.
@@ -194,11 +213,14 @@ void launch_rebuild_decide(const uint32_t *disp, uint32_t *disp_clear, uint32_t 
     launch_pdl(k_rebuild_decide, 1, 256, st, disp, disp_clear, rb, reps, n_rep, force, step_ctr, builds);
 }
 
-void launch_bin_next(const Buffers &b, const RepParams *reps, int n, int *count, int *tile_sum, int2 *cellrank,
-                     const uint32_t *rb, const uint32_t *any, cudaStream_t st, const DecideArgs &d)
+void launch_bin_next(const float4 *next_pos, const float4 *vel, const RepParams *reps, int n_rep, int n, int *count,
+                     int *tile_sum, int2 *cellrank, const uint32_t *rb, const uint32_t *any, cudaStream_t st,
+                     const DecideArgs &d)
 {
     if (n <= 0 && !d.disp) return;
-    launch_pdl(k_bin_next, std::max(1, (n + 255) / 256), 256, st, b, reps, n, count, tile_sum, cellrank, any, rb, d);
+    int g = std::max(1, (n + 2 * BIN_THREADS - 1) / (2 * BIN_THREADS));
+    if (d.disp) g = std::min(g, BIN_GRID_MAX);       // (of many replicas one nearly always rebuilds)
+    launch_pdl(k_bin_next, g, BIN_THREADS, st, next_pos, vel, reps, n_rep, n, count, tile_sum, cellrank, any, rb, d);
 }
 
 template <bool HALF>

@@ -210,12 +210,14 @@ struct SortSmallArgs {
 // ctas x SORT_SMALL_THREADS x SORT_SMALL_ITEMS particles
 int sort_small_ctas(int ns);
 void launch_sort_small(const SortSmallArgs &a, int ctas, cudaStream_t st);
-// cell and rank of the next predicted position of each particle of a
-// rebuilding replica (list mode, when any replica rebuilds; rb[r]: replica r
-// rebuilds, unless d.disp is set and the decision is taken here); a replica
-// that keeps its slots adds its particle count to its first cell
-void launch_bin_next(const Buffers &b, const RepParams *reps, int n, int *count, int *tile_sum, int2 *cellrank,
-                     const uint32_t *rb, const uint32_t *any, cudaStream_t st, const DecideArgs &d = DecideArgs{});
+// cell and rank of the next predicted position (next_pos, at the particles'
+// slots) of each particle of a rebuilding replica (list mode, when any replica
+// rebuilds; rb[r]: replica r rebuilds, unless d.disp is set and the decision is
+// taken here); a replica that keeps its slots adds its particle count to its first
+// cell
+void launch_bin_next(const float4 *next_pos, const float4 *vel, const RepParams *reps, int n_rep, int n, int *count,
+                     int *tile_sum, int2 *cellrank, const uint32_t *rb, const uint32_t *any, cudaStream_t st,
+                     const DecideArgs &d = DecideArgs{});
 void launch_list_build(const ListArgs &a, cudaStream_t st);
 // each membrane's reference point (ref_out[b]) from the load-order positions
 // x3 (three floats per particle) of a loaded state; max_nv, max_stride: the
