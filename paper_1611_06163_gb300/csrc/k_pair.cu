@@ -37,6 +37,8 @@ void launch_pair(const PairArgs &a, cudaStream_t st, int part)
         switch (a.ns) {
         case 1: launch_ns<1, false, false>(a, st, part); break;
         case 2: launch_ns<2, false, false>(a, st, part); break;
+        case 3: launch_ns<3, false, false>(a, st, part); break;
+        case 4: launch_ns<4, false, false>(a, st, part); break;
         default: launch_ns<0, false, false>(a, st, part); break;
         }
     }

@@ -1,7 +1,7 @@
 // Pair force + flux without any device allocation (tdpd_pair_forces_noalloc).
 //
 // Every scratch buffer this entry point needs -- the cell histogram and
-// offsets, the two sorted copies of the particle state, the slot maps -- lives
+// offsets, the sorted copy of the particle state, the slot maps -- lives
 // in one file-scope __device__ array of fixed size, g_noalloc_scratch, which
 // every GPU that loads the library holds until the process exits. The caller
 // supplies inputs and outputs; nothing is allocated or freed per call.
@@ -30,11 +30,12 @@ static_assert(NA_C % SCAN_TILE == 0, "the cell capacity is whole scan tiles");
 // Layout of the scratch array (only its size and offsets are used on the host).
 struct __align__(256) NoAllocLayout {
     RepParams params;
-    float4 pos[2][NA_N], vt[2][NA_N], vel[2][NA_N], frc[2][NA_N];
-    float C[2][NA_N * NA_S], Ct[2][NA_N * NA_S], Q[2][NA_N * NA_S];
+    float4 pos[NA_N], vt[NA_N], vel[NA_N], frc[NA_N];
+    float C[NA_N * NA_S], Ct[NA_N * NA_S], Q[NA_N * NA_S];
     float4 fext[NA_N];
     int inv[NA_N];
-    int2 cellrank[NA_N], keys[NA_N];
+    int2 cellrank[NA_N];
+    int keys[NA_N];
     int count[NA_C];
     int cell_start[NA_C + 4];
     int tile_sum[2][NA_TILES];
@@ -55,77 +56,116 @@ tdpd_status na_fail(tdpd_status code, const char *msg)
     return code;
 }
 
-// Copy the inputs into sorted-state buffer 0, clear what the binning counts
-// into, and set the step counter.
-__global__ void k_na_pack(RepParams P, int n, int ns, const float *__restrict__ pos,
-                          const float *__restrict__ vel, const float *__restrict__ conc,
-                          const int32_t *__restrict__ type, uint32_t step, NoAllocLayout *S)
+// The inputs sorted by cell, and by id within a cell, straight from the caller's
+// arrays: clear, bin, scan (k_scan), keys, place. Each launch is a few dependent
+// loads long, so fewer of them is what helps (12,000 particles: 16.8 us; with the
+// inputs first copied to a state buffer and gathered from there: 22.2; all of it in
+// one thread-block cluster: 27 with counters in the L2, 35 with counters and keys in
+// distributed shared memory, whose scattered atomics and loads are slower still).
+
+// What the binning counts into, the input check word and the call's parameters
+// (word by word: one thread's copy of the structure took 9 us).
+__global__ void k_na_clear(const __grid_constant__ RepParams P, int n, int cells, uint32_t step, NoAllocLayout *S)
 {
-    const int stride = gridDim.x * blockDim.x;
-    const int g0 = blockIdx.x * blockDim.x + threadIdx.x;
+    pdl_enter();
+    const int stride = gridDim.x * blockDim.x, g0 = blockIdx.x * blockDim.x + threadIdx.x;
+    static_assert(sizeof(RepParams) % 4 == 0, "copied by words");
+    for (int w = g0; w < (int)(sizeof(RepParams) / 4); w += stride)
+        reinterpret_cast<uint32_t *>(&S->params)[w] = reinterpret_cast<const uint32_t *>(&P)[w];
     if (g0 == 0) {
-        S->params = P;
-        S->err[0] = 0u;
+        S->err[0] = S->err[1] = 0u;
         S->step_ctr[0] = step;
+        S->cell_start[cells] = n;            // the end of the last scanned tile
     }
-    for (int c = g0; c < NA_C; c += stride) S->count[c] = 0;
-    // cells past the scanned tiles end at the particle count
-    for (int c = g0; c <= NA_C; c += stride) S->cell_start[c] = n;
+    for (int c = g0; c < cells; c += stride) S->count[c] = 0;
     for (int t = g0; t < 2 * NA_TILES; t += stride) S->tile_sum[t / NA_TILES][t % NA_TILES] = 0;
-    for (int k = g0; k < n; k += stride) {
-        // a type outside [0, n_types) is recorded (the outputs become NaN)
-        // and replaced by type 0, so that no table lookup leaves its range
-        int t = type[k];
-        if (t < 0 || t >= P.ntypes) {
-            atomicOr(&S->err[1], 4u);
-            t = 0;
-        }
-        const uint32_t w = (uint32_t)k | ((uint32_t)t << 24);
-        S->pos[0][k] = make_float4(pos[3 * k], pos[3 * k + 1], pos[3 * k + 2], __int_as_float((int)w));
-        S->vel[0][k] = make_float4(vel[3 * k], vel[3 * k + 1], vel[3 * k + 2], __int_as_float(0));
-        S->vt[0][k] = make_float4(vel[3 * k], vel[3 * k + 1], vel[3 * k + 2], __int_as_float(-1));
-        S->frc[0][k] = make_float4(0.f, 0.f, 0.f, 0.f);
-        for (int s = 0; s < ns; ++s) {
-            const float c = conc[(size_t)k * ns + s];
-            S->C[0][(size_t)k * ns + s] = c;
-            S->Ct[0][(size_t)k * ns + s] = c;
-            S->Q[0][(size_t)k * ns + s] = 0.f;
-        }
-    }
 }
 
-// Clear the input check word of this call (before k_na_pack may set it).
-__global__ void k_na_clear(NoAllocLayout *S)
+__global__ void k_na_bin(int n, const float *__restrict__ pos, NoAllocLayout *S)
 {
-    S->err[1] = 0u;
+    pdl_enter();
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    int c = -1;
+    if (k < n) {
+        c = cell_of(S->params, pos[3 * k], pos[3 * k + 1], pos[3 * k + 2]);
+        S->cellrank[k] = make_int2(c, atomicAdd(S->count + c, 1));
+    }
+    add_tile_count(S->tile_sum[0], c);
+}
+
+__global__ void k_na_keys(int n, NoAllocLayout *S)
+{
+    pdl_enter();
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= n) return;
+    const int2 cr = S->cellrank[k];
+    S->keys[S->cell_start[cr.x] + cr.y] = k;
+}
+
+// The particle of slot d's key goes to its rank by id inside its cell.
+__global__ void k_na_place(int n, int ns, const float *__restrict__ pos, const float *__restrict__ vel,
+                           const float *__restrict__ conc, const int32_t *__restrict__ type, NoAllocLayout *S)
+{
+    pdl_enter();
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= n) return;
+    const int k = S->keys[e], c = S->cellrank[k].x;
+    const int lo = S->cell_start[c], hi = S->cell_start[c + 1];
+    float4 p = make_float4(pos[3 * k], pos[3 * k + 1], pos[3 * k + 2], 0.f);
+    const float4 v = make_float4(vel[3 * k], vel[3 * k + 1], vel[3 * k + 2], __int_as_float(0));
+    float cs[NA_S];
+#pragma unroll
+    for (int s = 0; s < NA_S; ++s) cs[s] = s < ns ? conc[(size_t)k * ns + s] : 0.f;
+    int t = type[k], d = lo;
+    for (int q = lo; q < hi; ++q) d += S->keys[q] < k;
+    // a type outside [0, n_types) is recorded (the outputs become NaN)
+    // and replaced by type 0, so that no table lookup leaves its range
+    if (t < 0 || t >= S->params.ntypes) {
+        atomicOr(&S->err[1], 4u);
+        t = 0;
+    }
+    p.w = __int_as_float((int)((uint32_t)k | ((uint32_t)t << 24)));
+    S->pos[d] = p;
+    S->vel[d] = v;
+    S->vt[d] = make_float4(v.x, v.y, v.z, __int_as_float(-1));
+    S->frc[d] = make_float4(0.f, 0.f, 0.f, 0.f);
+    S->inv[k] = d;
+#pragma unroll
+    for (int s = 0; s < NA_S; ++s)
+        if (s < ns) {
+            S->C[(size_t)d * ns + s] = cs[s];
+            S->Ct[(size_t)d * ns + s] = cs[s];
+            S->Q[(size_t)d * ns + s] = 0.f;
+        }
 }
 
 // Load-order outputs; every output is NaN when an input type was out of
 // range or some force came out non-finite (the caller checks the outputs).
 __global__ void k_na_unpack(int n, int ns, const NoAllocLayout *S, float *force, float *flux)
 {
+    pdl_enter();
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= n) return;
     const bool bad = (S->err[0] | S->err[1]) != 0u;
     const float nan = __int_as_float(0x7fc00000);
     const int slot = S->inv[k];
-    const float4 f = S->frc[1][slot];
+    const float4 f = S->frc[slot];
     force[3 * k] = bad ? nan : f.x;
     force[3 * k + 1] = bad ? nan : f.y;
     force[3 * k + 2] = bad ? nan : f.z;
-    for (int s = 0; s < ns; ++s) flux[(size_t)k * ns + s] = bad ? nan : S->Q[1][(size_t)slot * ns + s];
+    for (int s = 0; s < ns; ++s) flux[(size_t)k * ns + s] = bad ? nan : S->Q[(size_t)slot * ns + s];
 }
 
-Buffers buffers(NoAllocLayout *S, int b)
+Buffers buffers(NoAllocLayout *S)
 {
     Buffers B;
-    B.pos = S->pos[b];
-    B.vt = S->vt[b];
-    B.vel = S->vel[b];
-    B.frc = S->frc[b];
-    B.C = S->C[b];
-    B.Ct = S->Ct[b];
-    B.Q = S->Q[b];
+    B.pos = S->pos;
+    B.vt = S->vt;
+    B.vel = S->vel;
+    B.frc = S->frc;
+    B.C = S->C;
+    B.Ct = S->Ct;
+    B.Q = S->Q;
     return B;
 }
 
@@ -184,15 +224,14 @@ extern "C" tdpd_status tdpd_pair_forces_noalloc(const tdpd_config *cfg, const fl
     const int ns = c.n_species;
     const RepParams P = build_rep_params(c, pair_coef, kappa, nc, m, 0, 0, n);
     cudaStream_t st = (cudaStream_t)stream;
-    k_na_clear<<<1, 1, 0, st>>>(S);
-    k_na_pack<<<64, 256, 0, st>>>(P, n, ns, pos, vel, conc, type, step, S);
-    const Buffers b0 = buffers(S, 0), b1 = buffers(S, 1);
+    const Buffers b1 = buffers(S);
     const RepParams *dP = &S->params;
-    const int n_tiles = (int)((ncell + SCAN_TILE - 1) / SCAN_TILE);
-    launch_bin_init(b0, dP, n, S->count, S->tile_sum[0], S->cellrank, st);
+    const int n_tiles = (int)((ncell + SCAN_TILE - 1) / SCAN_TILE), grid = (n + 255) / 256;
+    launch_pdl(k_na_clear, 16, 256, st, P, n, n_tiles * SCAN_TILE, step, S);
+    launch_pdl(k_na_bin, grid, 256, st, n, pos, S);
     launch_scan(S->count, S->cell_start, n_tiles, S->tile_sum[0], S->tile_sum[1], S->step_ctr, 0, st);
-    launch_scatter_keys(b0, S->cellrank, S->cell_start, S->keys, n, st);
-    launch_rank_gather(b0, b1, dP, S->keys, S->cellrank, S->cell_start, S->inv, n, ns, 0, st);
+    launch_pdl(k_na_keys, grid, 256, st, n, S);
+    launch_pdl(k_na_place, grid, 256, st, n, ns, pos, vel, conc, type, S);
     PairArgs a{};
     a.b = b1;
     a.fext = S->fext;
@@ -206,10 +245,14 @@ extern "C" tdpd_status tdpd_pair_forces_noalloc(const tdpd_config *cfg, const fl
     a.n = n;
     a.ns = ns;
     a.integrate = 0;
-    a.lpp = 1;
-    while (a.lpp < 8 && (long)n * a.lpp < 300000) a.lpp *= 2;
+    a.std_exp = c.s_f == 2.0f && c.s_c == 2.0f;
+    // lanes per particle: the stencil's 25 rows are split over them, and while the
+    // GPU is not full the rows left to each lane set the time (measured, pair
+    // kernel: 648 particles 34 us with 8 lanes, 18 with 32; 4,000: 22.5 with 8,
+    // 17.7 with 16, 19.8 with 32; 12,000: 24.5 with 8, 28.6 with 16)
+    a.lpp = n <= 1500 ? 32 : n <= 6000 ? 16 : 8;
     launch_pair(a, st);
-    k_na_unpack<<<(n + 255) / 256, 256, 0, st>>>(n, ns, S, force, flux);
+    launch_pdl(k_na_unpack, grid, 256, st, n, ns, S, force, flux);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return na_fail(TDPD_ECUDA, cudaGetErrorString(e));
     return TDPD_OK;
