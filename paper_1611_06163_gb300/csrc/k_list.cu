@@ -27,7 +27,11 @@
 
 namespace tdpd {
 
-constexpr int STRIPED_SPLIT_MAX = 60000;
+// Threads per particle of a striped build, and the particles up to which it has more
+// than one (measured, full lists of ten species, event time with 6 us of launch:
+// 27k particles 43 us with four threads, 46 with eight, 67 with one; 41k at a density
+// of 3: 48, 50, 59; 60k: 78, 80, 72; 286k: 213, 243, 169).
+constexpr int STRIPED_SPLIT = 4, STRIPED_SPLIT_MAX = 50000;
 
 __global__ void k_rebuild_decide(const uint32_t *__restrict__ disp, uint32_t *disp_clear, uint32_t *rb,
                                  const RepParams *__restrict__ reps, int n_rep, int force, uint32_t *step_ctr,
@@ -146,63 +150,88 @@ __global__ void __launch_bounds__(128) k_list_build(ListArgs A)
 }
 
 // The striped lists of the kernels with more than two species, B threads per
-// particle (a power of two): thread s takes the s-th of B consecutive parts of
-// the stencil's rows, counts its entries, and writes them after those of the
-// threads before it, so a list has the same order for every B. One thread walks
-// its rows once; several (small systems, where a thread per particle leaves the
-// GPU idle) walk them twice.
+// particle (a power of two), in the stencil's row order for every B. One thread
+// appends as it walks its rows; of several (small systems, where a thread per
+// particle leaves the GPU idle) each takes one of the next B rows, keeps up to
+// KEEP of its entries in shared memory until the B counts are known, and walks the
+// row a second time only for the entries beyond them (consecutive parts of the rows
+// per thread, each walked twice, 27k particles: 52 us against 43 -- the outer rows
+// are short and their threads idled).
 template <int M, bool HALF, int B>
 __global__ void __launch_bounds__(128) k_list_build_striped(ListArgs A)
 {
+    constexpr int KEEP = 8;
+    __shared__ int kept[B > 1 ? KEEP : 1][128];
     pdl_enter();
     if (!A.rb[A.n_rep]) return;                       // no replica rebuilds
     const int gt = blockIdx.x * blockDim.x + threadIdx.x;
     const int i = gt / B, sub = gt % B;
-    const bool valid = i < A.n;
-    const float4 pi = A.pos[valid ? i : 0];
-    const int rep = wbits(A.vel[valid ? i : 0].w);
-    bool need = valid && A.rb[rep] != 0u;
-    if (need && A.quar && A.quar[rep]) {              // quarantined: an empty list
+    if (i >= A.n) return;
+    const float4 pi = A.pos[i];
+    const int rep = wbits(A.vel[i].w);
+    if (!A.rb[rep]) return;
+    if (A.quar && A.quar[rep]) {                      // quarantined: an empty list
         if (sub == 0) A.nlc[i] = 0;
-        need = false;
+        return;
     }
     const RepParams &P = A.reps[rep];
-    const int m = M > 0 ? M : P.m_stencil, nrow = (2 * m + 1) * (2 * m + 1);
-    const int first = HALF ? nrow / 2 : 0, rows = nrow - first;
-    const int r0 = first + rows * sub / B, r1 = need ? first + rows * (sub + 1) / B : r0;
-    int e = 0, total = 0;
-    if (B > 1) {
-        int c = 0;
-        visit_rows<M, HALF, B == 1>(P, A.pos, A.cell_start, i, r0, r1, 1, pi, [&](const bool (&ok)[4], int) {
-            c += (int)ok[0] + (int)ok[1] + (int)ok[2] + (int)ok[3];
-        });
-        int x = c;
+    const int m = M > 0 ? M : P.m_stencil, nrow = (2 * m + 1) * (2 * m + 1), first = HALF ? nrow / 2 : 0;
+    // striped_row and striped_off by shifts (L is a power of two)
+    const int L = A.lpp, kl = __ffs(L) - 1, cap = A.cap;
+    int *list = A.nl + ((size_t)(i >> (5 - kl)) * (cap >> kl) * 32 + ((i & ((32 >> kl) - 1)) << kl));
+    auto off = [&](int e) { return ((e >> kl) << 5) + (e & (L - 1)); };
+    int total = 0;
+    if constexpr (B > 1) {
+        int *mine = &kept[0][threadIdx.x];
+        const unsigned group = ((1u << B) - 1u) << (threadIdx.x & 31 & ~(B - 1));   // the particle's lanes
+        for (int r0 = first; r0 < nrow; r0 += B) {
+            const int row = r0 + sub, end = min(row + 1, nrow);
+            int c = 0;
+            visit_rows<M, HALF, false>(P, A.pos, A.cell_start, i, row, end, 1, pi, [&](const bool (&ok)[4], int j0) {
 #pragma unroll
-        for (int o = 1; o < B; o <<= 1) {
-            const int v = __shfl_up_sync(0xffffffffu, x, o, B);
-            if (sub >= o) x += v;
+                for (int u = 0; u < 4; ++u)
+                    if (ok[u]) {
+                        if (c < KEEP) mine[c * 128] = j0 + u;
+                        ++c;
+                    }
+            });
+            int x = c;
+#pragma unroll
+            for (int o = 1; o < B; o <<= 1) {
+                const int v = __shfl_up_sync(group, x, o, B);
+                if (sub >= o) x += v;
+            }
+            const int e = total + x - c, room = cap - e;          // the row's first entry, entries left from it
+            for (int k = 0; k < min(min(c, KEEP), room); ++k) list[off(e + k)] = mine[k * 128];
+            if (c > KEEP && room > KEEP) {
+                int k = 0;
+                visit_rows<M, HALF, false>(P, A.pos, A.cell_start, i, row, end, 1, pi,
+                                           [&](const bool (&ok)[4], int j0) {
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+                        if (ok[u]) {
+                            if (k >= KEEP && k < room) list[off(e + k)] = j0 + u;
+                            ++k;
+                        }
+                });
+            }
+            total += __shfl_sync(group, x, B - 1, B);
         }
-        e = x - c;
-        total = __shfl_sync(0xffffffffu, x, B - 1, B);
-    }
-    if (B == 1 ? need : A.cap > 0) {
-        const int L = A.lpp, cap = A.cap;
-        int *list = A.nl + striped_row(i, L, cap / L);
-        int at = striped_off(e, L);
-        visit_rows<M, HALF, B == 1>(P, A.pos, A.cell_start, i, r0, r1, 1, pi, [&](const bool (&ok)[4], int j0) {
+    } else {
+        int at = 0;
+        visit_rows<M, HALF, true>(P, A.pos, A.cell_start, i, 0, 0, 1, pi, [&](const bool (&ok)[4], int j0) {
 #pragma unroll
             for (int u = 0; u < 4; ++u)
                 if (ok[u]) {
-                    if (e < cap) list[at] = j0 + u;
-                    ++e;
-                    at += (e & (L - 1)) ? 1 : 33 - L;
+                    if (total < cap) list[at] = j0 + u;
+                    ++total;
+                    at += (total & (L - 1)) ? 1 : 33 - L;
                 }
         });
-        if (B == 1) total = e;
     }
-    if (need && sub == 0) {
-        A.nlc[i] = A.cap > 0 ? min(total, A.cap) : total;
-        if (A.cap > 0 && total > A.cap) atomicOr(A.err + rep, 2u);
+    if (sub == 0) {
+        A.nlc[i] = cap > 0 ? min(total, cap) : total;
+        if (cap > 0 && total > cap) atomicOr(A.err + rep, 2u);
         A.xb[i] = pi;
     }
 }
@@ -250,9 +279,10 @@ static void launch_list_build_h(const ListArgs &a, int g, cudaStream_t st)
 template <int M, bool HALF>
 static void launch_striped(const ListArgs &a, cudaStream_t st)
 {
-    // eight threads per particle up to the particles that fill the GPU alone
+    // several threads per particle up to the particles that fill the GPU alone
     if (a.n <= STRIPED_SPLIT_MAX)
-        launch_pdl(k_list_build_striped<M, HALF, 8>, (int)((8L * a.n + 127) / 128), 128, st, a);
+        launch_pdl(k_list_build_striped<M, HALF, STRIPED_SPLIT>, (int)(((long)STRIPED_SPLIT * a.n + 127) / 128), 128,
+                   st, a);
     else
         launch_pdl(k_list_build_striped<M, HALF, 1>, (a.n + 127) / 128, 128, st, a);
 }

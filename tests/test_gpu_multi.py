@@ -15,8 +15,8 @@ from gpu_common import B, W, check_step, forces_vs_oracle, make
 pytestmark = pytest.mark.gpu
 
 
-def _box(ns, seed, L=6.0, types=2, flux=False, reaction=True, **kw):
-    d = W.fluid_box(L=L, rho=3.0, n_species=ns, seed=seed)
+def _box(ns, seed, L=6.0, types=2, flux=False, reaction=True, rho=3.0, **kw):
+    d = W.fluid_box(L=L, rho=rho, n_species=ns, seed=seed)
     rng = np.random.default_rng(seed)
     d['n_types'] = types
     for k in ('a', 'gamma', 'sigma'):
@@ -39,6 +39,14 @@ def test_forces_and_fluxes_match_oracle(ns, types, flux, lanes, mode):
     d = _box(ns, 500 + ns + lanes, types=types, flux=flux, lanes=lanes, pair_mode=mode)
     F, Q, Fo, Qo = forces_vs_oracle(d)
     check_step(F, Q, Fo, Qo, (ns, types, flux, lanes, mode))
+
+
+@pytest.mark.parametrize('mode', [1, 2])
+def test_dense_rows_match_oracle(mode):
+    """Rows of more entries than a build thread keeps (8) until it may write them."""
+    d = _box(3, 560, L=5.0, types=1, rho=16.0, lanes=4, pair_mode=mode)
+    F, Q, Fo, Qo = forces_vs_oracle(d)
+    check_step(F, Q, Fo, Qo, mode)
 
 
 def _run(h, steps, ns, reps=1):
