@@ -222,7 +222,7 @@ int tdpd_pair_mode(const tdpd_sys *s);
  * not set (tdpd_set_skin), commit times whole steps (16, list rebuilds
  * included) for the skins 0.2, 0.15, 0.25, 0.3 and 0.4, each with m = 2 and
  * m = 3 unless a replica sets cells_per_cutoff, and keeps the first within
- * 3 % of the fastest in that order; tuning_ms (may be NULL) receives up to
+ * 1.5 % of the fastest in that order; tuning_ms (may be NULL) receives up to
  * max_tuning of those times, in that order, and *n_tuning their count (0
  * when nothing was timed). No counterpart in the paper (it rebuilds its list
  * every few steps at a fixed radius). */
@@ -236,7 +236,7 @@ tdpd_status tdpd_list_shape(tdpd_sys *s, float *skin, int *cells_per_cutoff, flo
  * separated by the cluster barrier -- for systems of at most 32,768
  * particles (16,384 where only an 8-CTA cluster fits) and 1,048,576 cells,
  * where the chain's launches cost more than its work. Both give the same sorted order and the same bits. With 0,
- * commit times 16 steps of each (one graph replay each) where the cluster
+ * commit times 16 steps of each (graph replays) where the cluster
  * sort fits, and keeps it unless the chain is more than 3 % faster. Before
  * tdpd_commit; TDPD_EINVAL for another value, TDPD_ESTATE after commit;
  * commit fails with TDPD_EINVAL when 2 is set and the cluster sort does not

@@ -877,14 +877,58 @@ tdpd_status prepare_list(tdpd_sys *s)
 // each kernel, all on one stream)
 tdpd_status capture(tdpd_sys *s, int p, int len, cudaGraphExec_t *out, cudaEvent_t *ev = nullptr);
 
+// The time of 16 steps from the current state as they run later: replays of a
+// graph (of eight steps: building it costs as much as a small system's steps),
+// after two steps outside it (the parity is kept); of a small system up to eight
+// replays, since a short time varies with the rebuilds that fall into it. (Steps
+// launched one by one take at least the host's launch rate, longer than a small
+// system's step: the shapes of a 2,144-particle fluid then looked alike.)
+tdpd_status time_steps(tdpd_sys *s, float *ms)
+{
+    constexpr int LEN = 8;
+    static_assert(LEN % 2 == 0, "the parity is kept");
+    cudaStream_t st = exec_stream(s);
+    cudaGraphExec_t g = nullptr;
+    tdpd_status rc = capture(s, s->parity, LEN, &g);
+    if (rc) return rc;
+    cudaEvent_t e0 = nullptr, e1 = nullptr;
+    cudaError_t e = cudaEventCreate(&e0);
+    if (e == cudaSuccess) e = cudaEventCreate(&e1);
+    if (e == cudaSuccess) e = cudaGraphUpload(g, st);
+    for (int k = 0; k < 2 && e == cudaSuccess; ++k) {
+        enqueue_step(s, (s->parity + k) & 1, st);
+        e = cudaGetLastError();
+    }
+    float total = 0.f;
+    int n = 0;
+    for (int add = 2; add > 0;) {                     // two replays, then the others back to back
+        float t = 0.f;
+        if (e == cudaSuccess) e = cudaEventRecord(e0, st);
+        for (int k = 0; k < add && e == cudaSuccess; ++k) e = cudaGraphLaunch(g, st);
+        if (e == cudaSuccess) e = cudaEventRecord(e1, st);
+        if (e == cudaSuccess) e = cudaEventSynchronize(e1);
+        if (e == cudaSuccess) e = cudaEventElapsedTime(&t, e0, e1);
+        if (e != cudaSuccess) break;
+        total += t;
+        n += add;
+        add = n == 2 ? 2 * (int)std::min(3.f, 0.5f / std::max(t, 1e-3f)) : 0;
+    }
+    *ms = total * (16.f / LEN) / (float)std::max(n, 1);
+    cudaGraphExecDestroy(g);
+    if (e0) cudaEventDestroy(e0);
+    if (e1) cudaEventDestroy(e1);
+    if (e != cudaSuccess) return fail(s, TDPD_ECUDA, "timing of steps: %s", cudaGetErrorString(e));
+    return TDPD_OK;
+}
+
 // Pick the pair kernel's shape at commit by timing its forces-only mode
 // (idempotent apart from the next binning's counters) for each candidate:
 // the lanes per particle (1..32, or the pinned count) and, with neighbour
 // lists, the full shell (every pair from both sides) against the half shell
 // (each pair once, partner shares by fixed-point atomics), unless the mode is
 // pinned. The fastest of five timed launches per candidate; the candidates
-// within 10 % of the best are then timed as 16-step graph replays; the first
-// within 3 % of the best of those, half shell before full and fewer lanes
+// within 10 % of the best (30 % for the best of a shell) are then timed as whole
+// steps (time_steps); the first within 3 % of the best of those, half shell before full and fewer lanes
 // before more (they are no slower once the caches are cold, and near-equal
 // times would otherwise flip between runs). The state is then rebuilt with
 // the winner.
@@ -946,42 +990,27 @@ tdpd_status autotune(tdpd_sys *s)
     }
     float best = 1e30f;
     for (const auto &x : t) best = std::min(best, x.ms);
-    // the candidates within 10 % of the fastest launch are timed again as
-    // whole steps (16 of them as one graph replay, after one warm-up replay),
-    // which is what they will run as: in a short step the launch alone
-    // misjudges the half shell's finishing pass and the membrane join
+    // the candidates within 10 % of the fastest launch, and the fastest of the other
+    // shell if it is within 30 %, are timed again as whole steps, which is what they will run as: the
+    // launch alone misjudges the half shell's finishing pass and the membrane
+    // forces, which the full shell waits for and the half shell overlaps (a
+    // membrane in 12^3: 30 us a step against 39, pair launches 21 and 20)
     std::vector<Cand> fin;
-    for (const auto &x : t)
-        if (x.ms <= 1.10f * best) fin.push_back(x);
+    for (const auto &x : t) {
+        bool first = true;
+        for (const auto &y : t) first = first && (y.mode != x.mode || x.ms <= y.ms);
+        if (x.ms <= (first ? 1.30f : 1.10f) * best) fin.push_back(x);
+    }
     if (fin.size() > 1) {
-        constexpr int STEPS = 16;
         float bstep = 1e30f;
         for (Cand &x : fin) {
             s->lpp = x.lpp;
             s->half = x.mode == 2;
             tdpd_status rc;
-            if ((rc = reload_state(s))) {
+            if ((rc = reload_state(s)) || (rc = time_steps(s, &x.ms))) {
                 cudaEventDestroy(e0);
                 cudaEventDestroy(e1);
                 return rc;
-            }
-            cudaGraphExec_t g = nullptr;
-            if ((rc = capture(s, s->parity, STEPS, &g))) {
-                cudaEventDestroy(e0);
-                cudaEventDestroy(e1);
-                return rc;
-            }
-            cudaError_t e = cudaGraphLaunch(g, st);
-            if (e == cudaSuccess) e = cudaEventRecord(e0, st);
-            if (e == cudaSuccess) e = cudaGraphLaunch(g, st);
-            if (e == cudaSuccess) e = cudaEventRecord(e1, st);
-            if (e == cudaSuccess) e = cudaEventSynchronize(e1);
-            if (e == cudaSuccess) e = cudaEventElapsedTime(&x.ms, e0, e1);
-            cudaGraphExecDestroy(g);
-            if (e != cudaSuccess) {
-                cudaEventDestroy(e0);
-                cudaEventDestroy(e1);
-                return fail(s, TDPD_ECUDA, "autotune: %s", cudaGetErrorString(e));
             }
             bstep = std::min(bstep, x.ms);
         }
@@ -1128,95 +1157,69 @@ tdpd_status apply_shape(tdpd_sys *s, const Shape &sh)
 
 // Time the candidate shapes over a few whole steps each (the list rebuilds
 // they cause included) with the default lanes and pair mode, keep the first
-// within 3 % of the fastest (the default first), and leave it applied at
-// step 0 with the host's state loaded.
+// within 1.5 % of the fastest (the default first; time_steps repeats to 0.5 %),
+// and leave it applied at step 0 with the host's state loaded.
 tdpd_status tune_shape(tdpd_sys *s, const std::vector<Shape> &shapes)
 {
-    constexpr int STEPS = 16;
-    cudaStream_t st = exec_stream(s);
-    cudaEvent_t e0, e1;
-    CU(cudaEventCreate(&e0));
-    CU(cudaEventCreate(&e1));
     std::vector<float> t(shapes.size(), 1e30f);
-    tdpd_status rc = TDPD_OK;
-    for (size_t k = 0; k < shapes.size() && !rc; ++k) {
-        if ((rc = apply_shape(s, shapes[k]))) break;
-        int p = s->parity;
-        enqueue_step(s, p, st);                   // warm-up
-        p ^= 1;
-        cudaEventRecord(e0, st);
-        for (int it = 0; it < STEPS; ++it, p ^= 1) enqueue_step(s, p, st);
-        cudaEventRecord(e1, st);
-        cudaError_t e = cudaEventSynchronize(e1);
-        if (e == cudaSuccess) e = cudaEventElapsedTime(&t[k], e0, e1);
-        if (e == cudaSuccess) e = cudaGetLastError();
-        if (e != cudaSuccess) rc = fail(s, TDPD_ECUDA, "shape tuning: %s", cudaGetErrorString(e));
-    }
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
-    if (rc) return rc;
+    tdpd_status rc;
+    for (size_t k = 0; k < shapes.size(); ++k)
+        if ((rc = apply_shape(s, shapes[k])) || (rc = time_steps(s, &t[k]))) return rc;
     const float best = *std::min_element(t.begin(), t.end());
     size_t win = 0;
-    while (t[win] > 1.03f * best) ++win;
+    while (t[win] > 1.015f * best) ++win;
     s->shape_ms.assign(t.begin(), t.end());
     s->shape_win = (int)win;
     s->shape.skin = shapes[win].skin;
     s->shape.m = shapes[win].m;
     s->step = 0;
     if ((rc = apply_shape(s, shapes[win]))) return rc;
-    if (s->builds) CU(cudaMemsetAsync(s->builds, 0, sizeof(uint32_t) * s->reps.size(), st));
+    if (s->builds) CU(cudaMemsetAsync(s->builds, 0, sizeof(uint32_t) * s->reps.size(), exec_stream(s)));
     return TDPD_OK;
 }
 
+// CTAs of the one-cluster sort for the current shape; 0: it does not serve it.
+int sort_ctas_allowed(const tdpd_sys *s)
+{
+    const int ctas = s->NC <= SORT_SMALL_MAX_NC ? sort_small_ctas(s->ns) : 0;
+    return s->N <= ctas * SORT_SMALL_THREADS * SORT_SMALL_ITEMS ? ctas : 0;
+}
+
 // List mode: the sort of a step as one cluster launch or as the kernel chain.
-// Both give the same bits; unless the caller pinned one, time 16 steps of
-// each as one graph replay (after one warm-up replay) and keep the cluster
-// unless the chain is more than 3 % faster; then reload the host's state.
+// Both give the same bits; unless the caller pinned one, time steps with each and
+// keep the cluster unless the chain is more than 3 % faster; then reload the
+// host's state.
 tdpd_status tune_sort(tdpd_sys *s)
 {
     s->sort_ctas = 0;
     s->sort_ms.clear();
     if (!s->use_list || s->sort_fixed == 1) return TDPD_OK;
-    int ctas = s->NC <= SORT_SMALL_MAX_NC ? sort_small_ctas(s->ns) : 0;
-    const int max_n = ctas * SORT_SMALL_THREADS * SORT_SMALL_ITEMS;
-    if (s->N > max_n) ctas = 0;
-    if (s->sort_fixed == 2) {
-        if (!ctas)
-            return fail(s, TDPD_EINVAL, "the one-cluster sort needs at most %d particles and %d cells (here %d, %d) "
-                        "and a resident cluster of 8 or 16 CTAs", 16 * SORT_SMALL_THREADS * SORT_SMALL_ITEMS,
-                        SORT_SMALL_MAX_NC, s->N, s->NC);
-        s->sort_ctas = ctas;
-        return TDPD_OK;
-    }
-    if (!ctas) return TDPD_OK;
-    constexpr int STEPS = 16;
-    cudaStream_t st = exec_stream(s);
-    cudaEvent_t e0, e1;
-    CU(cudaEventCreate(&e0));
-    CU(cudaEventCreate(&e1));
+    const int ctas = sort_ctas_allowed(s);
+    if (s->sort_fixed == 2) s->sort_ctas = ctas;
+    if (s->sort_fixed == 2 || !ctas) return TDPD_OK;
     float t[2] = {1e30f, 1e30f};
-    tdpd_status rc = TDPD_OK;
-    for (int k = 0; k < 2 && !rc; ++k) {
+    tdpd_status rc;
+    for (int k = 0; k < 2; ++k) {
         s->sort_ctas = k == 0 ? ctas : 0;
-        cudaGraphExec_t g = nullptr;
-        if ((rc = capture(s, s->parity, STEPS, &g))) break;
-        cudaError_t e = cudaGraphLaunch(g, st);            // warm-up (an even count: same parity after)
-        if (e == cudaSuccess) e = cudaEventRecord(e0, st);
-        if (e == cudaSuccess) e = cudaGraphLaunch(g, st);
-        if (e == cudaSuccess) e = cudaEventRecord(e1, st);
-        if (e == cudaSuccess) e = cudaEventSynchronize(e1);
-        if (e == cudaSuccess) e = cudaEventElapsedTime(&t[k], e0, e1);
-        cudaGraphExecDestroy(g);
-        if (e != cudaSuccess) rc = fail(s, TDPD_ECUDA, "sort tuning: %s", cudaGetErrorString(e));
+        if ((k && (rc = init_state(s))) || (rc = time_steps(s, &t[k]))) return rc;
     }
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
-    if (rc) return rc;
     s->sort_ms.assign(t, t + 2);
     s->sort_ctas = t[0] <= 1.03f * t[1] ? ctas : 0;
     s->step = 0;
     if ((rc = init_state(s))) return rc;
-    if (s->builds) CU(cudaMemsetAsync(s->builds, 0, sizeof(uint32_t) * s->reps.size(), st));
+    if (s->builds) CU(cudaMemsetAsync(s->builds, 0, sizeof(uint32_t) * s->reps.size(), exec_stream(s)));
+    return TDPD_OK;
+}
+
+// The one-cluster sort against the limits of the shape that was kept.
+tdpd_status check_sort(tdpd_sys *s)
+{
+    const int ctas = s->use_list && s->sort_fixed != 1 ? sort_ctas_allowed(s) : 0;
+    if (s->use_list && s->sort_fixed == 2 && !ctas)
+        return fail(s, TDPD_EINVAL, "the one-cluster sort needs at most %d particles and %d cells (here %d, %d) "
+                    "and a resident cluster of 8 or 16 CTAs", 16 * SORT_SMALL_THREADS * SORT_SMALL_ITEMS,
+                    SORT_SMALL_MAX_NC, s->N, s->NC);
+    if (s->sort_fixed == 2 || !ctas) s->sort_ctas = ctas;
     return TDPD_OK;
 }
 
@@ -1501,9 +1504,11 @@ tdpd_status commit(tdpd_sys *s)
     CU(cudaStreamCreateWithFlags(&s->side, cudaStreamNonBlocking));
     CU(cudaEventCreateWithFlags(&s->fork, cudaEventDisableTiming));
     CU(cudaEventCreateWithFlags(&s->join, cudaEventDisableTiming));
+    // the sort first: lanes and shapes are then timed in steps as they will run
+    if ((rc = tune_sort(s))) return rc;
     if (!shapes.empty() && (rc = tune_shape(s, shapes))) return rc;
     if (s->lanes_fixed == 0 && (rc = autotune(s))) return rc;
-    if ((rc = tune_sort(s))) return rc;
+    if ((rc = check_sort(s))) return rc;
     const int nk = (int)step_kernels(s).size();
     for (int k = 0; k <= nk; ++k) CU(cudaEventCreate(&s->ev[k]));
     s->n_ev = nk + 1;
