@@ -769,14 +769,20 @@ long first_bad_particle(const tdpd_sys *s, const float *pos, const float *vel)
 void enqueue_init(tdpd_sys *s, cudaStream_t st, bool branch)
 {
     const int N = s->N, ns = s->ns;
-    cudaMemsetAsync(s->count, 0, sizeof(int) * (size_t)s->n_tiles * SCAN_TILE, st);
-    cudaMemsetAsync(s->tile_sum[0], 0, sizeof(int) * s->n_tiles, st);
-    cudaMemsetAsync(s->tile_sum[1], 0, sizeof(int) * s->n_tiles, st);
-    cudaMemsetAsync(s->errw, 0, sizeof(uint32_t) * s->reps.size(), st);
-    cudaMemsetAsync(s->quar, 0, sizeof(uint32_t) * s->reps.size(), st);
-    cudaMemsetAsync(s->fext, 0, sizeof(float4) * N, st);
-    launch_pack_state(s->d_in, s->d_wstat, s->buf[0], s->mx, s->mv, N, ns, st);
     branch = branch && s->n_rbc;
+    // the membranes' reference points need only the uploaded arrays: on the side
+    // stream they run beside the packing and the sort (one membrane: 26 us)
+    int max_stride = 0;
+    for (const RbcDev &D : s->h_rbcs) max_stride = std::max(max_stride, D.fan_stride);
+    if (branch) {
+        cudaEventRecord(s->fork, st);
+        cudaStreamWaitEvent(s->side, s->fork, 0);
+    }
+    launch_mem_ref(s->d_in, s->d_rbcs, s->d_fan, s->d_reps, s->d_ref[1], s->n_rbc, s->max_nv, max_stride,
+                   branch ? s->side : st);
+    const InitClear z{s->count, s->n_tiles * SCAN_TILE, s->tile_sum[0], s->tile_sum[1], s->n_tiles, s->errw, s->quar,
+                      s->use_list ? s->disp[1] : nullptr, (int)s->reps.size(), s->fext};
+    launch_pack_state(s->d_in, s->d_wstat, s->buf[0], s->mx, s->mv, N, ns, z, st);
     if (branch) {
         cudaEventRecord(s->fork, st);
         cudaStreamWaitEvent(s->side, s->fork, 0);
@@ -789,7 +795,6 @@ void enqueue_init(tdpd_sys *s, cudaStream_t st, bool branch)
     if (s->use_list) {
         launch_rank_gather(s->buf[0], s->buf[1], s->d_reps, s->keys, s->cellrank, s->cell_start, s->inv, N, ns, 0,
                            st, nullptr, 0, s->tile_sum[0], s->n_tiles, quarantine(s));
-        cudaMemsetAsync(s->disp[1], 0, sizeof(uint32_t) * s->reps.size(), st);
         // (the one- and two-species pair kernels build every lane's list
         // themselves, as on a step where every replica rebuilds)
         if (!pair_builds_lists(s)) launch_list_build(list_args(s, s->buf[1], s->rb_all, s->nl_cap), st);
@@ -807,16 +812,12 @@ void enqueue_init(tdpd_sys *s, cudaStream_t st, bool branch)
 }
 
 // Device part of loading a state whose load-order arrays are staged
-// (upload_in) or already in d_in: the membranes' reference points, then the
-// forces of the state.
+// (upload_in) or already in d_in.
 tdpd_status init_device(tdpd_sys *s, bool upload_in)
 {
     cudaStream_t st = exec_stream(s);
     tdpd_status rc;
     if (upload_in && (rc = upload(s, s->d_in, stage_in(s), (size_t)s->N * (6 + s->ns)))) return rc;
-    int max_stride = 0;
-    for (const RbcDev &D : s->h_rbcs) max_stride = std::max(max_stride, D.fan_stride);
-    launch_mem_ref(s->d_in, s->d_rbcs, s->d_fan, s->d_reps, s->d_ref[1], s->n_rbc, s->max_nv, max_stride, st);
     uint32_t *ctr = stage_ctr(s);
     ctr[0] = ctr[1] = ctr[2] = (uint32_t)s->step;        // sort / pair, membrane (by parity)
     if ((rc = upload(s, s->step_ctr, ctr, 3))) return rc;

@@ -8,6 +8,8 @@
 // the order in which atomics happened to land.
 #include <cooperative_groups.h>
 
+#include <algorithm>
+
 #include "launch.h"
 
 namespace tdpd {
@@ -564,11 +566,19 @@ namespace tdpd {
 // each) and C from the upload area, with each particle's fixed bits (id and
 // type, replica, membrane) from wstat; F and Q start at zero. Membrane
 // vertices also go to mx, mv (load order), where the membrane kernels read them.
+// The counters and status words of a loaded state are cleared here too (seven
+// memset nodes of the graph before: about 1.5 us each on a small system).
 __global__ void k_pack_state(const float *__restrict__ x3, const float *__restrict__ v3,
                              const float *__restrict__ c, const int4 *__restrict__ wstat, Buffers b,
-                             float4 *mx, float4 *mv, int n, int ns)
+                             float4 *mx, float4 *mv, int n, int ns, InitClear Z)
 {
-    const int g = blockIdx.x * blockDim.x + threadIdx.x;
+    const int g = blockIdx.x * blockDim.x + threadIdx.x, G = gridDim.x * blockDim.x;
+    for (int k = g; k < Z.n_count; k += G) Z.count[k] = 0;
+    for (int k = g; k < Z.n_tiles; k += G) Z.tile0[k] = Z.tile1[k] = 0;
+    for (int k = g; k < Z.n_rep; k += G) {
+        Z.err[k] = Z.quar[k] = 0u;
+        if (Z.disp) Z.disp[k] = 0u;
+    }
     if (g >= n) return;
     const int4 w = wstat[g];
     const float vx = v3[3 * (size_t)g], vy = v3[3 * (size_t)g + 1], vz = v3[3 * (size_t)g + 2];
@@ -580,6 +590,7 @@ __global__ void k_pack_state(const float *__restrict__ x3, const float *__restri
     if (w.z >= 0) {
         mx[g] = p;
         mv[g] = vt;
+        Z.fext[g] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
     b.frc[g] = make_float4(0.f, 0.f, 0.f, 0.f);
     for (int s = 0; s < ns; ++s) {
@@ -652,11 +663,11 @@ void launch_check_state(const float *x3, const float *v3, const int4 *wstat, con
 }
 
 void launch_pack_state(const float *in, const int4 *wstat, const Buffers &b, float4 *mx, float4 *mv, int n,
-                       int ns, cudaStream_t st)
+                       int ns, const InitClear &z, cudaStream_t st)
 {
-    if (n <= 0) return;
-    k_pack_state<<<(n + 255) / 256, 256, 0, st>>>(in, in + 3 * (size_t)n, in + 6 * (size_t)n, wstat, b, mx, mv,
-                                                  n, ns);
+    // a thread per particle, and enough of them for the counters of a sparse box
+    const int g = std::max({1, (n + 255) / 256, std::min(z.n_count / 1024, 608)});
+    k_pack_state<<<g, 256, 0, st>>>(in, in + 3 * (size_t)n, in + 6 * (size_t)n, wstat, b, mx, mv, n, ns, z);
 }
 
 }  // namespace tdpd

@@ -126,10 +126,22 @@ struct MemArgs {
     int n_rbc, max_nv;
 };
 
+// What the packing of a loaded state clears: the cell counters, both sets of tile
+// sums, the status and quarantine words, the next displacement maxima (null: cell
+// mode), and the membrane vertices' forces.
+struct InitClear {
+    int *count;
+    int n_count;
+    int *tile0, *tile1;
+    int n_tiles;
+    uint32_t *err, *quar, *disp;
+    int n_rep;
+    float4 *fext;
+};
 // in: x[3n], v[3n], C[n*ns] in load order; wstat: (id | type << 24, replica,
 // membrane or -1, 0) per particle; membrane vertices also to mx, mv
 void launch_pack_state(const float *in, const int4 *wstat, const Buffers &b, float4 *mx, float4 *mv, int n,
-                       int ns, cudaStream_t st);
+                       int ns, const InitClear &z, cudaStream_t st);
 // load-order device copies of a replica's slots [base, base + n) (any of the
 // outputs may be null); *bad set if the slot map is corrupt
 void launch_unpack_state(const Buffers &b, const int *inv, int base, int n, int ns, float *pos, float *vel,
