@@ -236,13 +236,16 @@ struct TrainSmem {
     float D2[HID][LDS_];
 };
 
+// PARTS: the launch takes every PARTS-th chunk, from `first` on, and (first > 0) adds
+// its sums to the row of the chunk before, so that a row of part holds PARTS chunks.
+template <int PARTS>
 __global__ void __launch_bounds__(TPB, 5) k_mlp_chunk(const float *__restrict__ params, const float *__restrict__ X,
                                                       const float *__restrict__ T, int n, float *part,
-                                                      float *loss_part)
+                                                      float *loss_part, int first, int nch)
 {
     __shared__ TrainSmem Q;
     NetSmem &S = Q.N;
-    const int mbr = blockIdx.y, c = blockIdx.x, nch = gridDim.x;
+    const int mbr = blockIdx.y, row = blockIdx.x, c = row * PARTS + first;
     const int t = threadIdx.x;
     const int s0 = 4 * (t & 7), to = t >> 3;
     {
@@ -269,7 +272,11 @@ __global__ void __launch_bounds__(TPB, 5) k_mlp_chunk(const float *__restrict__ 
         d3[1][r] = valid ? sc * e1 : 0.0f;
         err2 += valid ? e0 * e0 + e1 * e1 : 0.0f;
     }
-    float *out = part + ((size_t)mbr * nch + c) * NP;
+    float *out = part + ((size_t)mbr * gridDim.x + row) * NP;
+    auto put = [&](int k, float v) {
+        if (PARTS > 1 && first > 0) v += out[k];
+        out[k] = v;
+    };
     // sum of a value over the chunk's samples: the thread's four, then the
     // eight sample groups of the feature (lane bits 0-2)
     auto over_samples = [](float v) {
@@ -283,9 +290,9 @@ __global__ void __launch_bounds__(TPB, 5) k_mlp_chunk(const float *__restrict__ 
         const float l = over_samples(err2), b0 = over_samples((d3[0][0] + d3[0][1]) + (d3[0][2] + d3[0][3])),
                     b1 = over_samples((d3[1][0] + d3[1][1]) + (d3[1][2] + d3[1][3]));
         if (t == 0) {
-            loss_part[(size_t)mbr * nch + c] = l;
-            out[OB3] = b0;
-            out[OB3 + 1] = b1;
+            if (PARTS == 1 || c < nch) loss_part[(size_t)mbr * nch + c] = l;
+            put(OB3, b0);
+            put(OB3 + 1, b1);
         }
     }
 #pragma unroll
@@ -304,9 +311,9 @@ __global__ void __launch_bounds__(TPB, 5) k_mlp_chunk(const float *__restrict__ 
         a1 = over_samples(a1);
         const float b2 = over_samples((d2[0] + d2[1]) + (d2[2] + d2[3]));
         if (writer) {
-            out[OW3 + o] = a0;
-            out[OW3 + HID + o] = a1;
-            out[OB2 + o] = b2;
+            put(OW3 + o, a0);
+            put(OW3 + HID + o, a1);
+            put(OB2 + o, b2);
         }
     }
     __syncthreads();
@@ -346,9 +353,9 @@ __global__ void __launch_bounds__(TPB, 5) k_mlp_chunk(const float *__restrict__ 
                 w1[k] = over_samples(fmaf(d1[3], x.w, fmaf(d1[2], x.z, fmaf(d1[1], x.y, d1[0] * x.x))));
             }
             if (writer) {
-                out[OB1 + i] = b;
+                put(OB1 + i, b);
 #pragma unroll
-                for (int k = 0; k < IN; ++k) out[OW1 + i * IN + k] = w1[k];
+                for (int k = 0; k < IN; ++k) put(OW1 + i * IN + k, w1[k]);
             }
         }
     }
@@ -377,7 +384,7 @@ __global__ void __launch_bounds__(TPB, 5) k_mlp_chunk(const float *__restrict__ 
 #pragma unroll
         for (int q = 0; q < 4; ++q)
 #pragma unroll
-            for (int p = 0; p < 8; ++p) out[OW2 + (to + 16 * q) * HID + ii + 8 * p] = acc[q][p];
+            for (int p = 0; p < 8; ++p) put(OW2 + (to + 16 * q) * HID + ii + 8 * p, acc[q][p]);
     }
 }
 
@@ -460,14 +467,22 @@ void free_data(tdpd_mlp *m)
     m->cap = 0;
 }
 
+// Rows of the per-chunk gradient sums: a chunk each up to ROWS_MAX chunks (262,144
+// samples; 151 MB per member), above that four chunks each, which bounds the memory
+// at 144 bytes per sample and member (a row per chunk: 576).
+constexpr int ROWS_MAX = 8192;
+int grad_parts(int nch) { return nch <= ROWS_MAX ? 1 : 4; }
+
 tdpd_status alloc_data(tdpd_mlp *m, int n)
 {
     if (n <= m->cap) return TDPD_OK;
     cudaStreamSynchronize(m->st);
     free_data(m);
     const size_t M = m->members, nch = (size_t)(n + CH - 1) / CH;
+    // (fewer samples later may take more rows)
+    const size_t rows = nch <= (size_t)ROWS_MAX ? nch : std::max((nch + 3) / 4, (size_t)ROWS_MAX);
     float **bufs[] = {&m->X, &m->T, &m->loss_part, &m->gpart};
-    const size_t sizes[] = {(size_t)n * IN, (size_t)n * OUT, M * nch, M * nch * NP};
+    const size_t sizes[] = {(size_t)n * IN, (size_t)n * OUT, M * nch, M * rows * NP};
     for (int k = 0; k < 4; ++k) {
         void *p = nullptr;
         if (cudaMalloc(&p, sizes[k] * sizeof(float)) != cudaSuccess) {
@@ -505,7 +520,14 @@ tdpd_status pred_workspace(tdpd_mlp *m, size_t need)
 tdpd_status pass(tdpd_mlp *m, float lr, double *loss)
 {
     const int nch = (m->n + CH - 1) / CH;
-    launch_pdl(k_mlp_chunk, dim3(nch, m->members), TPB, m->st, m->params, m->X, m->T, m->n, m->gpart, m->loss_part);
+    const int parts = grad_parts(nch), rows = (nch + parts - 1) / parts;
+    if (parts == 1)
+        launch_pdl(k_mlp_chunk<1>, dim3(nch, m->members), TPB, m->st, m->params, m->X, m->T, m->n, m->gpart,
+                   m->loss_part, 0, nch);
+    else
+        for (int k = 0; k < parts; ++k)
+            launch_pdl(k_mlp_chunk<4>, dim3(rows, m->members), TPB, m->st, m->params, m->X, m->T, m->n, m->gpart,
+                       m->loss_part, k, nch);
     const int total = m->members * NP;
     float bc1 = 1.0f, bc2 = 1.0f;
     if (lr > 0.0f) {
@@ -513,7 +535,7 @@ tdpd_status pass(tdpd_mlp *m, float lr, double *loss)
         bc1 = (float)(1.0 - std::pow(0.9, (double)m->t));
         bc2 = (float)(1.0 - std::pow(0.999, (double)m->t));
     }
-    launch_pdl(k_mlp_reduce, (total + 31) / 32, 32 * RED_WARPS, m->st, m->gpart, nch, total, m->grad,
+    launch_pdl(k_mlp_reduce, (total + 31) / 32, 32 * RED_WARPS, m->st, m->gpart, rows, total, m->grad,
                lr > 0.0f ? 1 : 0, m->params, m->m, m->v, lr, 0.9f, 0.999f, 1e-8f, bc1, bc2);
     MCU(cudaGetLastError());
     if (loss) {

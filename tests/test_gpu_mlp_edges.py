@@ -50,3 +50,24 @@ def test_gradient_and_prediction_at_chunk_edges(n, members):
         assert np.abs(each[k] - y).max() < 1e-6 * np.abs(y).max(), k
     assert np.abs(mean - each.astype(np.float64).mean(0)).max() < 1e-6 * np.abs(mean).max()
     assert (spread == 0).all() if members == 1 else (spread > 0).any()
+
+
+def test_gradient_above_the_rows_of_one_chunk_each():
+    """Above 8,192 chunks a row of the chunk sums holds four of them; then fewer
+    samples, which take more rows, in the same allocation."""
+    bd = B()
+    P = S.init_params(77, 1)
+    h = bd.tdpd_mlp_create(1)
+    try:
+        bd.tdpd_mlp_set_params(h, P)
+        for n in (32 * 8192 + 33, 32 * 8192):
+            X, Y = _data(n, n)
+            bd.tdpd_mlp_set_data(h, X, Y)
+            loss, grad = bd.tdpd_mlp_loss_grad(h, 1)
+            st = mlp.Standardizer(X.astype(np.float64), Y.astype(np.float64))
+            lo, go = mlp.loss_grad(P[0], *(a.astype(np.float32).astype(np.float64) for a in
+                                           (st.x(X.astype(np.float64)), st.y(Y.astype(np.float64)))))
+            assert loss[0] == pytest.approx(lo, rel=1e-5)
+            assert normwise(grad[0], go) < 1e-5
+    finally:
+        bd.tdpd_mlp_destroy(h)
