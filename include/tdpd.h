@@ -333,7 +333,9 @@ tdpd_status tdpd_read_state_device(tdpd_sys *s, int replica, float *pos, float *
  * same configuration (same replicas, parameters, particle and membrane
  * counts, skin and lane count), which then continues exactly as the saved run
  * would have: the random numbers are keyed on the step, so a restart gives
- * the same bits. TDPD_EINVAL: the file cannot be opened, is not a checkpoint,
+ * the same bits (a version 2 file of a handle with more than two species or
+ * the random flux holds lists of another layout: it is accepted, and the lists
+ * are rebuilt at the next step). TDPD_EINVAL: the file cannot be opened, is not a checkpoint,
  * belongs to another configuration or is truncated (in the last case the
  * handle must be loaded again before use). Both commit an uncommitted handle
  * first, as tdpd_step does. */
