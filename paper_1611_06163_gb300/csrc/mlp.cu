@@ -213,10 +213,12 @@ __global__ void __launch_bounds__(TPB) k_mlp_stats(float *Y, Standard st, int me
         s += y;
         s2 += y * y;
     }
-    const double mu = s / members;
+    const double mu = s / members, size = fabs(mu);
     const double var = members > 1 ? fmax(0.0, (s2 - members * mu * mu) / (members - 1)) : 0.0;
     mean[e] = (float)mu;
-    rel[e] = (float)(sqrt(var) / fmax(fabs(mu), 1e-30));
+    // (compared, not fmax, which drops a NaN: a mean that is NaN has a NaN spread, for
+    // the callers trust a point by its small spread)
+    rel[e] = (float)(sqrt(var) / (size < 1e-30 ? 1e-30 : size));
 }
 
 // One training pass over a chunk of CH samples of one member: forward,

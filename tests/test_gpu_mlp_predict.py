@@ -1,0 +1,65 @@
+"""The prediction call of the surrogate where its statistics can
+go wrong: members or inputs that are not finite."""
+
+import numpy as np
+import pytest
+
+from workloads import surrogate as S
+from gpu_common import B
+
+pytestmark = pytest.mark.gpu
+
+
+def _points(n, seed):
+    rng = np.random.default_rng(seed)
+    return rng.uniform(0.1, 1.0, (n, 4)).astype(np.float32)
+
+
+def _handle(members, P=None, n=64):
+    bd = B()
+    h = bd.tdpd_mlp_create(members)
+    bd.tdpd_mlp_set_params(h, S.init_params(11, members) if P is None else P)
+    X = _points(n, 12)
+    bd.tdpd_mlp_set_data(h, X, np.stack([2 + X[:, 0] * X[:, 1], 3 + X[:, 3]], 1).astype(np.float32))
+    return h
+
+
+def _finite_predictions(h, X, members):
+    """(mean, spread, each) and the spread the members' outputs give in binary64."""
+    mean, spread, each = B().tdpd_mlp_predict(h, X, members)
+    e = each.astype(np.float64)
+    return mean, spread, each, e.std(0, ddof=1) / np.abs(e.mean(0))
+
+
+def test_a_nan_prediction_has_a_nan_spread():
+    """A caller trusts a point when its spread is small: the spread of a mean that
+    is NaN must not be. One input that is NaN touches its own row alone; one
+    diverged member (an output bias that is NaN) every row of that output."""
+    bd, members = B(), 4
+    X = _points(70, 13)
+    h = _handle(members)
+    try:
+        clean = bd.tdpd_mlp_predict(h, X, members)
+        Xn = X.copy()
+        Xn[33, 2] = np.nan
+        mean, spread, each, _ = _finite_predictions(h, Xn, members)
+    finally:
+        bd.tdpd_mlp_destroy(h)
+    assert np.isfinite(clean[1]).all() and (clean[1] > 0).all()
+    assert np.isnan(each[:, 33]).all() and np.isnan(mean[33]).all() and np.isnan(spread[33]).all()
+    rest = np.arange(70) != 33
+    for a, b in zip((mean, spread), clean[:2]):
+        assert np.array_equal(a[rest], b[rest])
+
+    P = S.init_params(11, members)
+    P[2, -1] = np.nan                       # the bias of the second output
+    h = _handle(members, P)
+    try:
+        mean, spread, each, want = _finite_predictions(h, X, members)
+    finally:
+        bd.tdpd_mlp_destroy(h)
+    assert np.isnan(mean[:, 1]).all() and np.isnan(spread[:, 1]).all()
+    assert np.isfinite(mean[:, 0]).all()
+    # the members' outputs are rounded to binary32 here: 2^-24 of the mean against
+    # a spread of per cents
+    assert np.abs(spread[:, 0] - want[:, 0]).max() < 1e-6
