@@ -512,7 +512,6 @@ PairArgs pair_args(tdpd_sys *s, const Buffers &b, int integrate, int *tile_sum, 
     a.klog = pair_klog(s->N, s->lpp);
     a.std_exp = 1;
     for (const HostRep &R : s->reps) {
-        a.nt = std::max(a.nt, (int)R.cfg.n_types);
         if (R.qr_ms > 0.0f) a.qr = 1;
         if (!(R.cfg.s_f == 2.0f && R.cfg.s_c == 2.0f)) a.std_exp = 0;
     }

@@ -178,10 +178,9 @@ __device__ __forceinline__ void epilogue(const PairArgs &A, const RepParams &P, 
         fz += sg * P.fbody[2];
     }
     if (reacts) {
-        const float rate = P.k_react * c_src;
         for (int s = 0; s < ns; ++s) {
-            if (s == P.r_src) q[s] -= rate;
-            if (s == P.r_dst) q[s] += rate;
+            if (s == P.r_src) q[s] = __fmaf_rn(-P.k_react, c_src, q[s]);
+            if (s == P.r_dst) q[s] = __fmaf_rn(P.k_react, c_src, q[s]);
         }
     }
     if (!isfinite(fx) || !isfinite(fy) || !isfinite(fz)) atomicOr(A.err + rep, 1u);
@@ -275,9 +274,9 @@ __device__ __forceinline__ void species_rows(const PairArgs &A, int base, int co
         const bool frozen = (P.frozen_mask >> ti) & 1u;
         float q = f, c = A.b.C[k];
         if (P.k_react != 0.0f && ((P.react_mask >> ti) & 1u)) {
-            const float rate = P.k_react * ct(p, P.r_src);
-            if (s == P.r_src) q -= rate;
-            if (s == P.r_dst) q += rate;
+            const float c_src = ct(p, P.r_src);
+            if (s == P.r_src) q = __fmaf_rn(-P.k_react, c_src, q);
+            if (s == P.r_dst) q = __fmaf_rn(P.k_react, c_src, q);
         }
         if (A.integrate && !frozen) {
             c = __fmaf_rn(P.hdt, A.b.Q[k] + q, c);    // C_{k+1}

@@ -39,6 +39,15 @@ struct MultiSmem {
     float c[32 * NS], qs[32 * NS];   // predicted concentrations and own flux sums
 };
 
+// A replica with one type and no partner shares sums its fluxes without kappa and
+// scales them at the end; its own parameters decide, so that it takes the same
+// formula alone and beside other replicas.
+template <bool HALF, bool QR>
+__device__ __forceinline__ bool scaled_flux(const RepParams &P)
+{
+    return !HALF && P.ntypes == 1 && !(QR && P.qr_coef > 0.0f);
+}
+
 constexpr float ROUND_MAGIC = 12582912.0f;    // 1.5 x 2^23: x + M - M rounds x to an integer
 
 }  // namespace
@@ -91,9 +100,6 @@ __global__ void __launch_bounds__(128, NS <= 4 ? 6 : NS <= 10 ? 5 : 3) k_pair_mu
     float q[NS];
 #pragma unroll
     for (int s = 0; s < NS; ++s) q[s] = 0.0f;
-    // with one type and no partner shares the fluxes are summed without kappa
-    // and scaled at the end
-    const bool scaled = !HALF && !QR && A.nt == 1;
     int qhead = 0, qcount = 0;
     const int capb = A.cap / L;
     const int *ptr = A.nl + striped_row(base + grp, L, capb) + sub;
@@ -113,7 +119,7 @@ __global__ void __launch_bounds__(128, NS <= 4 ? 6 : NS <= 10 ? 5 : 3) k_pair_mu
         const RepParams &P = A.reps[rep];
         const float Lx = P.L[0], Ly = P.L[1], Lz = P.L[2], iLx = P.inv_L[0], iLy = P.inv_L[1], iLz = P.inv_L[2];
         const float rc2 = P.rc2, rcc2 = P.rcc2, inv_rcc = P.inv_rcc, s_c = P.s_c;
-        const bool sc2 = P.sc_is2;
+        const bool sc2 = P.sc_is2, random = QR && P.qr_coef > 0.0f, scaled = scaled_flux<HALF, QR>(P);
         const float *kap_row = P.kappa + (int)((uint32_t)wbits(xi.w) >> 24) * P.ntypes * ns;
         for (int e = 0; e < nmax; e += L) {
             // the next trip's positions and the indices of the one after are in
@@ -176,7 +182,6 @@ __global__ void __launch_bounds__(128, NS <= 4 ? 6 : NS <= 10 ? 5 : 3) k_pair_mu
                     // one pair normal per species (the (cos, sin) pair of
                     // stream 6 + s/2), signed by the id order so that
                     // zeta_ji = -zeta_ij
-                    const bool random = QR && P.qr_coef > 0.0f;
                     const uint32_t idi = (uint32_t)wbits(xi.w) & ID_MASK, idj = wj & ID_MASK;
                     float amp = 0.0f;
                     if (random) amp = (idi < idj ? 1.0f : -1.0f) * P.qr_coef * sqrtf(wdc) * P.inv_sqrt_dt;
@@ -185,13 +190,19 @@ __global__ void __launch_bounds__(128, NS <= 4 ? 6 : NS <= 10 ? 5 : 3) k_pair_mu
                     for (int s = 0; s < NS; ++s) {
                         if (RT && s >= ns) break;
                         const float ks = __ldg(kap + s);
-                        float f = -(ks * wdc * (ci[s] - cj[s]));
+                        // (rounded explicitly: the same bits in every form)
+                        const float kw = __fmul_rn(ks, wdc), dc = __fsub_rn(ci[s], cj[s]);
+                        float f;
                         if (random) {
                             if ((s & 1) == 0)
                                 z = normal2(pair_bits(idi, idj, P.seed_lo, P.seed_hi, step_ctr + P.step0, 6u + (uint32_t)(s >> 1)));
-                            f += amp * sqrtf(fmaxf(ks * (ci[s] + cj[s]), 0.0f)) * ((s & 1) ? z.y : z.x);
+                            const float fr = amp * sqrtf(fmaxf(ks * (ci[s] + cj[s]), 0.0f)) * ((s & 1) ? z.y : z.x);
+                            f = __fmaf_rn(-kw, dc, fr);
+                            q[s] = __fadd_rn(q[s], f);
+                        } else {
+                            f = -__fmul_rn(kw, dc);
+                            q[s] = __fmaf_rn(-kw, dc, q[s]);
                         }
-                        q[s] += f;
                         if (HALF) acc_add(A.accQ + (size_t)j0 * ns + s, -f, ACC_Q_SCALE, ACC_Q_LIMIT, A.err + rep);
                     }
                 }
@@ -244,7 +255,8 @@ __global__ void __launch_bounds__(128, NS <= 4 ? 6 : NS <= 10 ? 5 : 3) k_pair_mu
                                   [&](int p) { return make_int2(W.li[p].rep, (int)W.li[p].wi); },
                                   [&](int p, int s, size_t) {
                                       const float f = M.qs[p * NS + s];
-                                      return scaled ? f * __ldg(A.reps[W.li[p].rep].kappa + s) : f;
+                                      const RepParams &R = A.reps[W.li[p].rep];
+                                      return scaled_flux<HALF, QR>(R) ? __fmul_rn(f, __ldg(R.kappa + s)) : f;
                                   },
                                   [&](int p, int s) { return M.c[p * NS + s]; });
         record_displacement(A.disp_next, rep, disp2, live, lane);

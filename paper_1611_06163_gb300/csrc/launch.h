@@ -57,7 +57,6 @@ struct PairArgs {
     int integrate;               // 0: forces only (commit / set_state); 1: full step
     int lpp;                     // lanes per particle: 1, 2, 4, 8, 16 or 32
     int qr;                      // some replica has the random flux (general kernel)
-    int nt;                      // largest number of types of a replica
     int klog;                    // striped lists: 2^klog rounds of 32 / lpp particles per warp
     int std_exp;                 // every replica has s_f = 2 and s_c = 2 (kernels with them fixed)
     // neighbour-list mode (nl != nullptr): partners from the list instead of

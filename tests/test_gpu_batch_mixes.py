@@ -1,0 +1,71 @@
+"""A replica gives the same bits in a batch as alone (at equal lanes and pair mode)
+when the other replicas of the batch differ in the number of types, in the random
+flux or in the weight exponents, so that the batch takes other forms of the kernels
+than the replica alone."""
+
+import numpy as np
+import pytest
+
+from gpu_common import B, W, make
+
+pytestmark = pytest.mark.gpu
+
+PLAIN, TYPES, FLUX, FLUX_TYPES, SOFT = dict(), dict(types=2), dict(flux=True), dict(types=2, flux=True), dict(s_f=0.41)
+
+
+def _box(ns, seed, L, types=1, flux=False, s_f=2.0):
+    d = W.fluid_box(L=L, rho=3.0, n_species=ns, seed=seed)
+    rng = np.random.default_rng(seed)
+    d['n_types'], d['s_f'] = types, s_f
+    for k in ('a', 'gamma', 'sigma'):
+        d[k] = np.full((types, types), d[k][0, 0], np.float32)
+    kap = rng.uniform(0.2, 2.0, (types, types, ns)).astype(np.float32)
+    d['kappa'] = (0.5 * (kap + kap.transpose(1, 0, 2))).astype(np.float32)
+    d['particles']['type'] = rng.integers(0, types, d['particles']['pos'].shape[0]).astype(np.int32)
+    if ns > 1:
+        d['reaction'] = dict(k=0.3, src=0, dst=ns - 1, types=1)
+    if flux:
+        d['random_flux'] = dict(m_s=0.05, rho=3.0)
+    return d
+
+
+def _results(h, ns, replicas):
+    bd = B()
+    out = [[] for _ in range(replicas)]
+    for steps in (0, 1, 11):                  # the loaded state, a step, rebuilds of the lists
+        if steps:
+            bd.tdpd_step(h, steps)
+        bd.tdpd_sync(h)
+        for r in range(replicas):
+            out[r] += list(bd.tdpd_read_state(h, r, ns) + bd.tdpd_read_forces(h, r, ns))
+    return out
+
+
+@pytest.mark.parametrize('mix', [(PLAIN, TYPES), (PLAIN, FLUX), (TYPES, FLUX_TYPES), (FLUX, TYPES), (PLAIN, SOFT)])
+@pytest.mark.parametrize('ns, lanes, mode', [(3, 4, 1), (3, 1, 2), (10, 1, 1), (10, 8, 1), (10, 8, 2), (16, 2, 1),
+                                             (2, 2, 0), (3, 8, 0)])
+def test_batch_equals_alone_in_mixed_batches(mix, ns, lanes, mode):
+    """mode 0: cell mode (skin 0)."""
+    bd = B()
+    skin, mode = (0.2, mode) if mode else (0.0, 1)
+    ds = [dict(_box(ns, 50 + k + 7 * ns, 5.1 + k, **kw), lanes=lanes, pair_mode=mode, skin=skin)
+          for k, kw in enumerate(mix)]
+    alone = []
+    for d in ds:
+        h = make(d)
+        alone.append(_results(h, ns, 1)[0])
+        bd.tdpd_destroy(h)
+    hs = [bd.create_from(d) for d in ds]
+    b = bd.tdpd_batch_create(hs)
+    for h in hs:
+        bd.tdpd_destroy(h)
+    try:
+        bd.tdpd_set_lanes(b, lanes)
+        bd.tdpd_set_pair_mode(b, mode)
+        bd.tdpd_set_skin(b, skin)
+        bd.tdpd_commit(b)
+        for k, got in enumerate(_results(b, ns, len(ds))):
+            for x, y in zip(got, alone[k]):
+                assert np.array_equal(x, y), k
+    finally:
+        bd.tdpd_destroy(b)
