@@ -134,8 +134,7 @@ tdpd_status tdpd_set_reaction(tdpd_sys *s, float k, int src, int dst, uint32_t t
  * + on the side of the smaller id, so each pair exchanges solute. m_s = 0
  * (the default) leaves it out, as the paper does (m_s << m). rho is the
  * particle number density of the model, m_s the solute mass. Before commit;
- * TDPD_EINVAL for negative or non-finite values. Handles that use it run the
- * general (any species count) pair kernel. */
+ * TDPD_EINVAL for negative or non-finite values. */
 tdpd_status tdpd_set_random_flux(tdpd_sys *s, float m_s, float rho);
 
 /* Body force profile: 0 (default) the configuration's body force everywhere;
@@ -333,9 +332,9 @@ tdpd_status tdpd_read_state_device(tdpd_sys *s, int replica, float *pos, float *
  * same configuration (same replicas, parameters, particle and membrane
  * counts, skin and lane count), which then continues exactly as the saved run
  * would have: the random numbers are keyed on the step, so a restart gives
- * the same bits (a version 2 file of a handle with more than two species or
- * the random flux holds lists of another layout: it is accepted, and the lists
- * are rebuilt at the next step). TDPD_EINVAL: the file cannot be opened, is not a checkpoint,
+ * the same bits (a file whose lists have another layout -- version 2 of a
+ * handle with more than two species, version 3 of one with one or two -- is
+ * accepted, and the lists are rebuilt at the next step). TDPD_EINVAL: the file cannot be opened, is not a checkpoint,
  * belongs to another configuration or is truncated (in the last case the
  * handle must be loaded again before use). Both commit an uncommitted handle
  * first, as tdpd_step does. */

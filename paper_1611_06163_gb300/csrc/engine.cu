@@ -455,19 +455,13 @@ MemArgs mem_args(tdpd_sys *s, int ref_in, int inc)
     return m;
 }
 
-// List mode with one or two species (and no random flux): the pair kernel
-// (its one- and two-species forms) builds the lists of rebuilding replicas
-// itself; the forms for more species and for the random flux read striped lists
-// (list_striped.cuh) that a kernel of their own builds before them.
-bool pair_builds_lists(const tdpd_sys *s)
-{
-    if (!s->use_list || s->ns > 2) return false;
-    for (const HostRep &R : s->reps)
-        if (R.qr_ms > 0.0f) return false;
-    return true;
-}
-
-bool striped_lists(const tdpd_sys *s) { return s->use_list && !pair_builds_lists(s); }
+// List mode with one or two species: the pair kernel builds the lists of
+// rebuilding replicas itself; the kernels for more species read striped lists
+// (list_striped.cuh) that a kernel of their own builds before them. The species
+// count alone decides, which all replicas of a batch share: a replica's list, and
+// with it the order of its sums, is the same alone and in any batch.
+bool pair_builds_lists(const tdpd_sys *s) { return s->use_list && s->ns <= 2; }
+bool striped_lists(const tdpd_sys *s) { return s->use_list && s->ns > 2; }
 
 // Rounds per warp of the kernels on striped lists (a power of two up to the
 // lanes, so that a warp holds at most 32 particles): as many as leave the GPU
@@ -1995,6 +1989,9 @@ tdpd_status config_hash(tdpd_sys *s, uint64_t *out)
     return TDPD_OK;
 }
 
+// 2: list mode also saves the other buffer; 3: the same with striped lists
+uint32_t ckp_version(const tdpd_sys *s) { return striped_lists(s) ? 3 : 2; }
+
 // (device pointer, bytes) of every saved array, in file order
 std::vector<std::pair<void *, size_t>> ckp_arrays(tdpd_sys *s, int parity, size_t nl_ints, uint32_t version)
 {
@@ -2020,10 +2017,10 @@ std::vector<std::pair<void *, size_t>> ckp_arrays(tdpd_sys *s, int parity, size_
         v.push_back({s->disp[0], 4 * nr});
         v.push_back({s->disp[1], 4 * nr});
         v.push_back({s->builds, 4 * nr});
-        // (striped lists are not read from a version 2 file, which holds one
-        // list per lane: null, and the next step rebuilds them)
-        const bool striped = striped_lists(s), skip = striped && version < 3;
-        v.push_back({skip ? nullptr : s->nlc, 4 * N * (striped && !skip ? 1 : (size_t)s->lpp)});
+        // (lists of the other layout -- one per lane in version 2, one per particle in
+        // version 3 -- are not read: null, and the next step rebuilds them)
+        const bool skip = version != ckp_version(s);
+        v.push_back({skip ? nullptr : s->nlc, 4 * N * (version >= 3 ? 1 : (size_t)s->lpp)});
         v.push_back({s->xb, 16 * N});
         v.push_back({skip ? nullptr : s->nl, 4 * nl_ints});
     }
@@ -2043,9 +2040,6 @@ size_t nl_used_ints(const tdpd_sys *s)
 {
     return s->use_list ? list_ints(s->N, striped_lists(s), s->lpp, s->nl_cap) : 0;
 }
-
-// 2: list mode also saves the other buffer; 3: the same with striped lists
-uint32_t ckp_version(const tdpd_sys *s) { return striped_lists(s) ? 3 : 2; }
 
 tdpd_status tdpd_save(tdpd_sys *s, const char *path)
 {
@@ -2096,7 +2090,8 @@ tdpd_status tdpd_load(tdpd_sys *s, const char *path)
     uint64_t h = 0;
     if ((rc = config_hash(s, &h))) { std::fclose(f); return rc; }
     if (H.N != s->N || H.NC != s->NC || H.ns != s->ns || H.n_rep != (int)s->reps.size() || H.n_rbc != s->n_rbc ||
-        (H.use_list != 0) != s->use_list || H.n_tiles != s->n_tiles || H.cfg_hash != h || H.version > ckp_version(s)) {
+        (H.use_list != 0) != s->use_list || H.n_tiles != s->n_tiles || H.cfg_hash != h ||
+        (!s->use_list && H.version != ckp_version(s))) {
         std::fclose(f);
         return fail(s, TDPD_EINVAL, "checkpoint of another configuration (particles, cells, species, replicas, "
                                     "membranes, list mode or parameters differ)");
@@ -2116,9 +2111,9 @@ tdpd_status tdpd_load(tdpd_sys *s, const char *path)
         std::fclose(f);
         return fail(s, TDPD_EINVAL, "corrupt checkpoint header");
     }
-    // the list layout follows the capacity of the saved run (lists of the other
-    // layout are skipped, and the capacity stays)
-    const bool skip = s->use_list && H.version < ckp_version(s);
+    // the list capacity follows the saved run (lists of the other layout are skipped,
+    // and the capacity stays)
+    const bool skip = s->use_list && H.version != ckp_version(s);
     const bool recapture = s->use_list && !skip && H.nl_cap != s->nl_cap;
     if (s->use_list) {
         const size_t need = list_ints(s->N, H.version >= 3, s->lpp, H.nl_cap);

@@ -16,9 +16,9 @@
 //
 // k_list_build counts the entries at commit; on a rebuild step and for a loaded
 // state the pair kernel's one- and two-species forms build their own lanes' lists
-// (list_lane.cuh). The kernels for more species and for the random flux read
-// lists of another layout (list_striped.cuh), one per particle, which
-// k_list_build_striped builds before them.
+// (list_lane.cuh). The kernels for more species read lists of another layout
+// (list_striped.cuh), one per particle, which k_list_build_striped builds before
+// them.
 #include <algorithm>
 
 #include "launch.h"

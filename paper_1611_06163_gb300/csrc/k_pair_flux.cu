@@ -1,4 +1,4 @@
-// The list-mode pair kernels with the random flux (Eq. 7).
+// The list-mode pair kernels with the random flux (Eq. 7) for more than two species.
 #include "k_pair_multi.cuh"
 
 namespace tdpd {

@@ -1,5 +1,5 @@
-// The pair kernels (included by k_pair.cu and k_pair_std.cu, which
-// instantiate them).
+// The pair kernels (included by k_pair.cu, k_pair_std.cu and k_pair_flux_lane.cu,
+// which instantiate them).
 //
 // Pairwise tDPD force (Eq. 3) and Fickian flux (Eq. 6), fused with the
 // velocity-Verlet corrector. Two ways to find the partners:
@@ -308,9 +308,11 @@ __device__ __forceinline__ void record_displacement(uint32_t *disp_next, int rep
 
 }  // namespace
 
-template <int NS, int LPP, bool LIST, bool HALF, bool STD>
+// QR: the random flux of Eq. 7 (the replicas that have it).
+template <int NS, int LPP, bool LIST, bool HALF, bool STD, bool QR>
 __global__ void __launch_bounds__(128, 6) k_pair(PairArgs A)
 {
+    static_assert(!LIST || NS == 1 || NS == 2, "more species have their own list-mode kernel (k_pair_multi.cuh)");
     static_assert(LIST || !HALF, "the half shell needs neighbour lists");
     pdl_enter();
     __shared__ WarpSmem smem[4];
@@ -388,41 +390,43 @@ __global__ void __launch_bounds__(128, 6) k_pair(PairArgs A)
         const float w = 1.0f - r * inv_rcc;
         const float wdc = sc2 ? w * w : __powf(w, s_c);
         const int tj = (int)(wj >> 24);
+        // (the terms that every form shares are rounded explicitly: a replica gives
+        // the same bits whichever form its batch takes)
         if (NS == 1) {
             float kap = kr[0];
             kap = tj == 1 ? kr[1] : kap;
             kap = tj == 2 ? kr[2] : kap;
             kap = tj == 3 ? kr[3] : kap;
-            const float qd = kap * wdc * (ci[0] - cj0);
-            const float qn = q[0] - qd;
+            const float kw = __fmul_rn(kap, wdc), dc = __fsub_rn(ci[0], cj0);
+            const float qn = __fmaf_rn(-kw, dc, q[0]);
             q[0] = inc ? qn : q[0];
-            if (HALF && inc) acc_add(A.accQ + j, qd, ACC_Q_SCALE, ACC_Q_LIMIT, A.err + rep);
+            if (HALF && inc) acc_add(A.accQ + j, __fmul_rn(kw, dc), ACC_Q_SCALE, ACC_Q_LIMIT, A.err + rep);
         } else if (inc) {
             const float *kap = kap_row + tj * ns;
-            const float qd0 = kap[0] * wdc * (ci[0] - cj0);
-            q[0] -= qd0;
-            if (HALF) acc_add(A.accQ + (size_t)j * ns, qd0, ACC_Q_SCALE, ACC_Q_LIMIT, A.err + rep);
-            for (int s = 1; s < ns; ++s) {
-                const float qd = kap[s] * wdc * (ci[s] - Ct[(size_t)j * ns + s]);
-                q[s] -= qd;
-                if (HALF) acc_add(A.accQ + (size_t)j * ns + s, qd, ACC_Q_SCALE, ACC_Q_LIMIT, A.err + rep);
+            for (int s = 0; s < ns; ++s) {
+                const float cj = s == 0 ? cj0 : Ct[(size_t)j * ns + s];
+                const float kw = __fmul_rn(kap[s], wdc), dc = __fsub_rn(ci[s], cj);
+                q[s] = __fmaf_rn(-kw, dc, q[s]);
+                if (HALF)
+                    acc_add(A.accQ + (size_t)j * ns + s, __fmul_rn(kw, dc), ACC_Q_SCALE, ACC_Q_LIMIT, A.err + rep);
             }
-            if (NS == 0 && P.qr_coef > 0.0f) {
-                // random flux (Eq. 7): eps w_RC zeta / sqrt(dt), eps^2 =
-                // m_s^2 kappa rho (C_i + C_j), w_RC = w_DC^(1/2) (Eq. 8); one
-                // pair normal per species (the (cos, sin) pair of stream
-                // 6 + s/2), signed by the id order so that zeta_ji = -zeta_ij
-                const uint32_t idi = wi & ID_MASK, idj = wj & ID_MASK;
-                const float amp = (idi < idj ? 1.0f : -1.0f) * P.qr_coef * sqrtf(wdc) * P.inv_sqrt_dt;
-                float2 z = make_float2(0.f, 0.f);
-                for (int s = 0; s < ns; ++s) {
-                    if ((s & 1) == 0)
-                        z = normal2(pair_bits(idi, idj, P.seed_lo, P.seed_hi, step_ctr + P.step0, 6u + (uint32_t)(s >> 1)));
-                    const float cs = ci[s] + (s == 0 ? cj0 : Ct[(size_t)j * ns + s]);
-                    const float qr = amp * sqrtf(fmaxf(kap[s] * cs, 0.0f)) * ((s & 1) ? z.y : z.x);
-                    q[s] += qr;
-                    if (HALF) acc_add(A.accQ + (size_t)j * ns + s, -qr, ACC_Q_SCALE, ACC_Q_LIMIT, A.err + rep);
-                }
+        }
+        if (QR && inc && P.qr_coef > 0.0f) {
+            // random flux (Eq. 7): eps w_RC zeta / sqrt(dt), eps^2 =
+            // m_s^2 kappa rho (C_i + C_j), w_RC = w_DC^(1/2) (Eq. 8); one
+            // pair normal per species (the (cos, sin) pair of stream
+            // 6 + s/2), signed by the id order so that zeta_ji = -zeta_ij
+            const float *kap = kap_row + tj * ns;
+            const uint32_t idi = wi & ID_MASK, idj = wj & ID_MASK;
+            const float amp = (idi < idj ? 1.0f : -1.0f) * P.qr_coef * sqrtf(wdc) * P.inv_sqrt_dt;
+            float2 z = make_float2(0.f, 0.f);
+            for (int s = 0; s < ns; ++s) {
+                if ((s & 1) == 0)
+                    z = normal2(pair_bits(idi, idj, P.seed_lo, P.seed_hi, step_ctr + P.step0, 6u + (uint32_t)(s >> 1)));
+                const float cs = ci[s] + (s == 0 ? cj0 : Ct[(size_t)j * ns + s]);
+                const float qr = amp * sqrtf(fmaxf(kap[s] * cs, 0.0f)) * ((s & 1) ? z.y : z.x);
+                q[s] += qr;
+                if (HALF) acc_add(A.accQ + (size_t)j * ns + s, -qr, ACC_Q_SCALE, ACC_Q_LIMIT, A.err + rep);
             }
         }
         const bool push = near && r2 < rc2;
@@ -444,18 +448,14 @@ __global__ void __launch_bounds__(128, 6) k_pair(PairArgs A)
     if constexpr (LIST) {
         // the lane's list, UNR_LIST entries per trip (index loads, then partner
         // loads, then the visits in list order); separations by minimum image
-        if constexpr (NS == 1 || NS == 2) {
-            // rebuild step: this lane's list first (the lists are only ever
-            // read by the lane that owns them, so no other thread waits);
-            // the kernels for more species keep the separate list build
-            // (the build's registers would cost them more than the launch)
-            if (A.rb && live && A.rb[rep]) {
-                ListArgs L{};
-                L.pos = pos; L.vel = A.b.vel; L.reps = A.reps; L.cell_start = A.cell_start; L.rb = A.rb;
-                L.nl = A.nl_w; L.nlc = A.nlc_w; L.xb = A.xb_w; L.err = A.err; L.n = A.n; L.lpp = LPP; L.cap = A.cap;
-                if (A.m2) build_lane<LPP, 2, HALF>(L, gt, i, sub, pi, rep);
-                else build_lane<LPP, 0, HALF>(L, gt, i, sub, pi, rep);
-            }
+        // rebuild step: this lane's list first (the lists are only ever
+        // read by the lane that owns them, so no other thread waits)
+        if (A.rb && live && A.rb[rep]) {
+            ListArgs L{};
+            L.pos = pos; L.vel = A.b.vel; L.reps = A.reps; L.cell_start = A.cell_start; L.rb = A.rb;
+            L.nl = A.nl_w; L.nlc = A.nlc_w; L.xb = A.xb_w; L.err = A.err; L.n = A.n; L.lpp = LPP; L.cap = A.cap;
+            if (A.m2) build_lane<LPP, 2, HALF>(L, gt, i, sub, pi, rep);
+            else build_lane<LPP, 0, HALF>(L, gt, i, sub, pi, rep);
         }
         // (plain loads: on a rebuild step this thread has just written them)
         const int *nl = A.nl + (size_t)(gt >> 5) * A.cap * 32 + (gt & 31);
@@ -675,34 +675,36 @@ void launch_pair_finish(const PairArgs &a, cudaStream_t st);
 // the pair kernels with the standard exponents (k_pair_std.cu; one or two
 // species, no random flux)
 void launch_pair_std(const PairArgs &a, cudaStream_t st, int part);
+// list mode with the random flux for one or two species (k_pair_flux_lane.cu)
+void launch_pair_flux_lane(const PairArgs &a, cudaStream_t st, int part);
 
-template <int NS, bool LIST, bool HALF, bool STD>
+template <int NS, bool LIST, bool HALF, bool STD, bool QR>
 static void launch_lanes(const PairArgs &a, cudaStream_t st)
 {
     const int t = 128;
     const long threads = (long)a.n * a.lpp;
     const int g = (int)((threads + t - 1) / t);
     switch (a.lpp) {
-    case 1: launch_pdl(k_pair<NS, 1, LIST, HALF, STD>, g, t, st, a); break;
-    case 2: launch_pdl(k_pair<NS, 2, LIST, HALF, STD>, g, t, st, a); break;
-    case 4: launch_pdl(k_pair<NS, 4, LIST, HALF, STD>, g, t, st, a); break;
-    case 8: launch_pdl(k_pair<NS, 8, LIST, HALF, STD>, g, t, st, a); break;
-    case 16: launch_pdl(k_pair<NS, 16, LIST, HALF, STD>, g, t, st, a); break;
-    default: launch_pdl(k_pair<NS, 32, LIST, HALF, STD>, g, t, st, a); break;
+    case 1: launch_pdl(k_pair<NS, 1, LIST, HALF, STD, QR>, g, t, st, a); break;
+    case 2: launch_pdl(k_pair<NS, 2, LIST, HALF, STD, QR>, g, t, st, a); break;
+    case 4: launch_pdl(k_pair<NS, 4, LIST, HALF, STD, QR>, g, t, st, a); break;
+    case 8: launch_pdl(k_pair<NS, 8, LIST, HALF, STD, QR>, g, t, st, a); break;
+    case 16: launch_pdl(k_pair<NS, 16, LIST, HALF, STD, QR>, g, t, st, a); break;
+    default: launch_pdl(k_pair<NS, 32, LIST, HALF, STD, QR>, g, t, st, a); break;
     }
 }
 
-template <int NS, bool LIST, bool STD>
+template <int NS, bool LIST, bool STD, bool QR = false>
 static void launch_ns(const PairArgs &a, cudaStream_t st, int part)
 {
     if constexpr (LIST) {
         if (a.half) {
-            if (part & PAIR_WALK) launch_lanes<NS, true, true, STD>(a, st);
+            if (part & PAIR_WALK) launch_lanes<NS, true, true, STD, QR>(a, st);
             if (part & PAIR_FINISH) launch_pair_finish(a, st);
             return;
         }
     }
-    if (part & PAIR_WALK) launch_lanes<NS, LIST, false, STD>(a, st);
+    if (part & PAIR_WALK) launch_lanes<NS, LIST, false, STD, QR>(a, st);
 }
 
 }  // namespace tdpd

@@ -1,7 +1,6 @@
-// The list-mode pair kernel for more than two species and for the random flux:
-// pairwise tDPD force (Eq. 3) and the fluxes of every species (Eq. 6, and Eq. 7),
-// full or half shell, as k_pair (k_pair_impl.cuh), with another division of the
-// work.
+// The list-mode pair kernel for more than two species: pairwise tDPD force (Eq. 3)
+// and the fluxes of every species (Eq. 6, and Eq. 7), full or half shell, as k_pair
+// (k_pair_impl.cuh), with another division of the work.
 //
 // A partner here is a row of concentrations beside its position: with one
 // particle per lane (k_pair's layout) 32 lanes gather 32 rows that share no
@@ -14,7 +13,9 @@
 // entries s, s + L, ... in list order and a butterfly adds the lanes: the sum
 // depends on the list and on L alone, not on K or on the particles that share the
 // warp. (One and two species keep k_pair: there the rows are short, and the
-// additional instructions per entry cost more than the gathers.)
+// additional instructions per entry cost more than the gathers; with the random flux
+// too, so that a replica's sums have one order whether or not another replica of its
+// batch has the flux.)
 //
 // Ten species, 286k particles, full shell: 236 us (k_pair's layout 344). Ten
 // species with the random flux, 41k particles, half shell: 108 us and 17 for the

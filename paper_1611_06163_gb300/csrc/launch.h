@@ -56,7 +56,7 @@ struct PairArgs {
     int ns;                      // species (runtime value for the generic path)
     int integrate;               // 0: forces only (commit / set_state); 1: full step
     int lpp;                     // lanes per particle: 1, 2, 4, 8, 16 or 32
-    int qr;                      // some replica has the random flux (general kernel)
+    int qr;                      // some replica has the random flux
     int klog;                    // striped lists: 2^klog rounds of 32 / lpp particles per warp
     int std_exp;                 // every replica has s_f = 2 and s_c = 2 (kernels with them fixed)
     // neighbour-list mode (nl != nullptr): partners from the list instead of
@@ -64,7 +64,7 @@ struct PairArgs {
     const int *nl;               // [warps][cap][32] partner slots per lane
     const int *nlc;              // [n*lpp] entries per lane
     int cap;                     // entries per lane
-    // (more than two species or the random flux: one list per particle,
+    // (more than two species: one list per particle,
     // list_striped.cuh, cap its entries, nlc [n])
     const float4 *xb;            // [n] positions at the last list build
     uint32_t *disp_next;         // [n_rep] max squared displacement (float bits) of the next positions
@@ -184,8 +184,8 @@ void launch_rank_gather(const Buffers &cur, const Buffers &nxt, const RepParams 
 // pass (nothing in full-shell and cell mode), or both
 constexpr int PAIR_WALK = 1, PAIR_FINISH = 2, PAIR_ALL = 3;
 void launch_pair(const PairArgs &a, cudaStream_t st, int part = PAIR_ALL);
-// its list-mode forms (the walk alone) for more than two species and with the
-// random flux
+// its list-mode forms (the walk alone) for more than two species, without and with
+// the random flux
 void launch_pair_multi(const PairArgs &a, cudaStream_t st);
 void launch_pair_flux(const PairArgs &a, cudaStream_t st);
 // rb[r] = the displacement of replica r exceeds half its skin (or force);

@@ -1,12 +1,15 @@
 """A replica gives the same bits in a batch as alone (at equal lanes and pair mode)
 when the other replicas of the batch differ in the number of types, in the random
 flux or in the weight exponents, so that the batch takes other forms of the kernels
-than the replica alone."""
+than the replica alone. Forces and fluxes of the forms that only the mixes reach
+against the oracle, and checkpoints whose lists have the other layout."""
+
+import struct
 
 import numpy as np
 import pytest
 
-from gpu_common import B, W, make
+from gpu_common import B, W, check_step, forces_vs_oracle, make
 
 pytestmark = pytest.mark.gpu
 
@@ -42,8 +45,9 @@ def _results(h, ns, replicas):
 
 
 @pytest.mark.parametrize('mix', [(PLAIN, TYPES), (PLAIN, FLUX), (TYPES, FLUX_TYPES), (FLUX, TYPES), (PLAIN, SOFT)])
-@pytest.mark.parametrize('ns, lanes, mode', [(3, 4, 1), (3, 1, 2), (10, 1, 1), (10, 8, 1), (10, 8, 2), (16, 2, 1),
-                                             (2, 2, 0), (3, 8, 0)])
+@pytest.mark.parametrize('ns, lanes, mode', [(1, 1, 1), (1, 4, 2), (1, 32, 1), (2, 4, 1), (2, 1, 2), (2, 32, 2),
+                                             (3, 4, 1), (3, 1, 2), (10, 1, 1), (10, 8, 1), (10, 8, 2), (16, 2, 1),
+                                             (1, 2, 0), (2, 2, 0), (3, 8, 0)])
 def test_batch_equals_alone_in_mixed_batches(mix, ns, lanes, mode):
     """mode 0: cell mode (skin 0)."""
     bd = B()
@@ -69,3 +73,50 @@ def test_batch_equals_alone_in_mixed_batches(mix, ns, lanes, mode):
                 assert np.array_equal(x, y), k
     finally:
         bd.tdpd_destroy(b)
+
+
+@pytest.mark.parametrize('ns, types, lanes, mode', [(1, 1, 1, 1), (1, 3, 4, 2), (1, 2, 32, 1), (2, 2, 2, 2),
+                                                    (2, 1, 16, 1), (2, 3, 1, 2)])
+def test_random_flux_of_few_species_matches_oracle(ns, types, lanes, mode):
+    d = dict(_box(ns, 90 + ns + lanes, 6.0, types=types, flux=True), lanes=lanes, pair_mode=mode)
+    F, Q, Fo, Qo = forces_vs_oracle(d)
+    check_step(F, Q, Fo, Qo, (ns, types, lanes, mode))
+
+
+def test_checkpoint_with_lists_per_particle_is_accepted(tmp_path):
+    """A version 3 file (one list per particle, here left at zero) of a handle with two
+    species and the random flux, whose lists are per lane: accepted, and the lists
+    are rebuilt at the next step."""
+    bd = B()
+    ns, lanes = 2, 4
+    d = dict(_box(ns, 96, 7.0, flux=True), lanes=lanes, pair_mode=1, skin=0.2)
+    h = make(d)
+    path = str(tmp_path / 'c')
+    bd.tdpd_step(h, 7)
+    bd.tdpd_save(h, path)
+    raw = open(path, 'rb').read()
+    size = struct.calcsize('<8sI11i')
+    size += -size % 8 + 24
+    head = list(struct.unpack_from('<8sI11i', raw))
+    tail = struct.unpack_from('<qQQ', raw, size - 24)
+    N, lpp = head[2], head[7]
+    assert head[1] == 2 and N == bd.tdpd_num_particles(h) and lpp == lanes
+    body, nl, nlc = raw[size:], 4 * tail[2], 4 * N * lanes
+    xb = body[-(nl + 16 * N):-nl]
+    front = body[:len(body) - nl - 16 * N - nlc]
+    cap3 = 24
+    ints = (N * lanes + 31) // 32 * 32 * (cap3 // lanes)
+    head[1], head[9] = 3, cap3
+    pad = b'\0' * (size - 24 - struct.calcsize('<8sI11i'))
+    open(path, 'wb').write(struct.pack('<8sI11i', *head) + pad + struct.pack('<qQQ', tail[0], tail[1], ints) + front +
+                           b'\0' * (4 * N) + xb + b'\0' * (4 * ints))
+    want = _results(h, ns, 1)[0]
+    bd.tdpd_load(h, path)
+    got = _results(h, ns, 1)[0]
+    bd.tdpd_destroy(h)
+    # the same state; after a step its rebuilt lists change the order of the sums
+    for k, (x, y) in enumerate(zip(got, want)):
+        if k < 5:
+            assert np.array_equal(x, y)
+        elif k < 10:
+            assert np.abs(x - y).max() <= 1e-5 * np.abs(y).max()
