@@ -10,6 +10,7 @@
 
 #include <cmath>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <string>
 #include <vector>
@@ -440,8 +441,11 @@ struct tdpd_mlp {
     Standard sd = {};
     float *base = nullptr;      // one allocation: params, m, v, grad, the first workspace
     // prediction workspace, kept between calls up to PRED_KEEP floats: inputs,
-    // then mean, relative spread and the members' outputs
+    // then mean, relative spread and the members' outputs. One call at a time uses
+    // it, from its copy of the inputs to the read of its results (pred_use), so that
+    // threads may predict with one handle; the calls share the handle's stream anyway
     float *pred = nullptr, *pred_own = nullptr;
+    std::mutex pred_use;
     size_t pred_floats = 0;
     bool have_data = false;
     cudaStream_t st = nullptr;
@@ -511,7 +515,7 @@ tdpd_status pred_workspace(tdpd_mlp *m, size_t need)
         cudaGetLastError();
         return mfail(TDPD_ENOMEM, "tdpd_mlp_predict: device allocation failed");
     }
-    if (m->pred_own) cudaFree(m->pred_own);       // (every call waits for its work)
+    if (m->pred_own) cudaFree(m->pred_own);       // (every call waits for its work before it lets go)
     m->pred = m->pred_own = (float *)d;
     m->pred_floats = need;
     return TDPD_OK;
@@ -672,8 +676,10 @@ tdpd_status tdpd_mlp_predict(tdpd_mlp *m, int n, const float *X, float *mean, fl
     const size_t need = in + ens + each;
     // a call beyond the kept workspace allocates for itself
     const bool keep = need <= PRED_KEEP;
+    std::unique_lock<std::mutex> use(m->pred_use, std::defer_lock);
     float *d = nullptr;
     if (keep) {
+        use.lock();
         tdpd_status rc = pred_workspace(m, need);
         if (rc) return rc;
         d = m->pred;

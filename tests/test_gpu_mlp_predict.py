@@ -1,5 +1,8 @@
-"""The prediction call of the surrogate where its statistics can
-go wrong: members or inputs that are not finite."""
+"""The prediction call of the surrogate where its statistics and its workspace can
+go wrong: members or inputs that are not finite, calls of several threads on one
+handle."""
+
+import threading
 
 import numpy as np
 import pytest
@@ -63,3 +66,32 @@ def test_a_nan_prediction_has_a_nan_spread():
     # the members' outputs are rounded to binary32 here: 2^-24 of the mean against
     # a spread of per cents
     assert np.abs(spread[:, 0] - want[:, 0]).max() < 1e-6
+
+
+def test_threads_share_a_handle():
+    """Calls of several threads on one handle (as before the handle kept its
+    workspace), the sizes on both sides of what comes with it."""
+    bd, members = B(), 2
+    h = _handle(members)
+    sets = [_points(n, 20 + n) for n in (300, 5462, 1000, 9000, 301, 20000, 5463, 2048)]
+    right = []
+
+    def work(k):
+        for _ in range(40):
+            got = bd.tdpd_mlp_predict(h, sets[k], members)
+            right.append(all(np.array_equal(a, b) for a, b in zip(got, want[k])))
+
+    try:
+        want = []
+        for X in sets:
+            g = _handle(members)
+            want.append(bd.tdpd_mlp_predict(g, X, members))
+            bd.tdpd_mlp_destroy(g)
+        threads = [threading.Thread(target=work, args=(k,)) for k in range(len(sets))]
+        for t in threads:
+            t.start()
+        for t in threads:
+            t.join()
+    finally:
+        bd.tdpd_mlp_destroy(h)
+    assert len(right) == 40 * len(sets) and all(right)
