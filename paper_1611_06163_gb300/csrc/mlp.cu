@@ -447,7 +447,9 @@ struct tdpd_mlp {
     float *pred = nullptr, *pred_own = nullptr;
     std::mutex pred_use;
     size_t pred_floats = 0;
-    bool have_data = false;
+    // samples to train on in X and T; a standardisation to predict with (it outlives
+    // the samples when a larger set does not fit)
+    bool have_data = false, have_std = false;
     cudaStream_t st = nullptr;
     std::vector<void *> data_allocs;
 };
@@ -470,7 +472,9 @@ void free_data(tdpd_mlp *m)
 {
     for (void *p : m->data_allocs) cudaFree(p);
     m->data_allocs.clear();
-    m->cap = 0;
+    m->cap = m->n = 0;
+    m->X = m->T = m->loss_part = m->gpart = nullptr;
+    m->have_data = false;
 }
 
 // Rows of the per-chunk gradient sums: a chunk each up to ROWS_MAX chunks (262,144
@@ -479,6 +483,8 @@ void free_data(tdpd_mlp *m)
 constexpr int ROWS_MAX = 8192;
 int grad_parts(int nch) { return nch <= ROWS_MAX ? 1 : 4; }
 
+// Buffers for n samples, the gradient rows first (the largest). On failure the handle
+// has no samples.
 tdpd_status alloc_data(tdpd_mlp *m, int n)
 {
     if (n <= m->cap) return TDPD_OK;
@@ -487,11 +493,12 @@ tdpd_status alloc_data(tdpd_mlp *m, int n)
     const size_t M = m->members, nch = (size_t)(n + CH - 1) / CH;
     // (fewer samples later may take more rows)
     const size_t rows = nch <= (size_t)ROWS_MAX ? nch : std::max((nch + 3) / 4, (size_t)ROWS_MAX);
-    float **bufs[] = {&m->X, &m->T, &m->loss_part, &m->gpart};
-    const size_t sizes[] = {(size_t)n * IN, (size_t)n * OUT, M * nch, M * rows * NP};
+    float **bufs[] = {&m->gpart, &m->X, &m->T, &m->loss_part};
+    const size_t sizes[] = {M * rows * NP, (size_t)n * IN, (size_t)n * OUT, M * nch};
     for (int k = 0; k < 4; ++k) {
         void *p = nullptr;
         if (cudaMalloc(&p, sizes[k] * sizeof(float)) != cudaSuccess) {
+            cudaGetLastError();                   // (not the next call's error)
             free_data(m);
             return mfail(TDPD_ENOMEM, "tdpd_mlp: device allocation failed");
         }
@@ -639,7 +646,7 @@ tdpd_status tdpd_mlp_set_data(tdpd_mlp *m, int n, const float *X, const float *Y
     MCU(cudaMemcpyAsync(m->T, ys.data(), ys.size() * sizeof(float), cudaMemcpyHostToDevice, m->st));
     MCU(cudaStreamSynchronize(m->st));
     m->n = n;
-    m->have_data = true;
+    m->have_data = m->have_std = true;
     return TDPD_OK;
 }
 
@@ -671,7 +678,7 @@ tdpd_status tdpd_mlp_train(tdpd_mlp *m, int steps, float lr, double *loss)
 tdpd_status tdpd_mlp_predict(tdpd_mlp *m, int n, const float *X, float *mean, float *rel_spread, float *member_out)
 {
     if (!m || n < 1 || !X || !mean) return mfail(TDPD_EINVAL, "tdpd_mlp_predict: bad arguments");
-    if (!m->have_data) return mfail(TDPD_ESTATE, "tdpd_mlp_predict: no standardisation (set data first)");
+    if (!m->have_std) return mfail(TDPD_ESTATE, "tdpd_mlp_predict: no standardisation (set data first)");
     const size_t N = (size_t)n, in = N * IN, ens = 2 * N * OUT, each = (size_t)m->members * N * OUT;
     const size_t need = in + ens + each;
     // a call beyond the kept workspace allocates for itself

@@ -1,6 +1,6 @@
 """The prediction call of the surrogate where its statistics and its workspace can
 go wrong: members or inputs that are not finite, calls of several threads on one
-handle."""
+handle; and the handle after an allocation that failed."""
 
 import threading
 
@@ -95,3 +95,30 @@ def test_threads_share_a_handle():
     finally:
         bd.tdpd_mlp_destroy(h)
     assert len(right) == 40 * len(sets) and all(right)
+
+
+def test_samples_that_do_not_fit_leave_a_usable_handle():
+    """Two thousand million samples with 64 members need 18 TB of gradient rows: the
+    allocation fails before the samples are read. Training then has no data (a status,
+    no launch), prediction keeps the standardisation it had, and a set that fits trains
+    as on a new handle."""
+    bd, members = B(), 64
+    h, g = _handle(members), _handle(members)
+    X = _points(50, 14)
+    Y = np.stack([2 + X[:, 1], 3 + X[:, 2] * X[:, 3]], 1).astype(np.float32)
+    try:
+        before = bd.tdpd_mlp_predict(h, X, members)
+        assert bd.STATUS[bd.lib.tdpd_mlp_set_data(h, 2_000_000_000, bd._ptr(X), bd._ptr(Y))] == 'ENOMEM'
+        for call in (lambda: bd.tdpd_mlp_train(h, 1, 1e-3, members), lambda: bd.tdpd_mlp_loss_grad(h, members)):
+            with pytest.raises(bd.TdpdError) as e:
+                call()
+            assert bd.STATUS[e.value.status] == 'ESTATE'
+        for a, b in zip(before, bd.tdpd_mlp_predict(h, X, members)):
+            assert np.array_equal(a, b)
+        for x in (h, g):
+            bd.tdpd_mlp_set_data(x, X, Y)
+        for a, b in zip(bd.tdpd_mlp_loss_grad(h, members), bd.tdpd_mlp_loss_grad(g, members)):
+            assert np.array_equal(a, b)
+    finally:
+        bd.tdpd_mlp_destroy(h)
+        bd.tdpd_mlp_destroy(g)
