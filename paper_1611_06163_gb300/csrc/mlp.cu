@@ -690,8 +690,9 @@ tdpd_status tdpd_mlp_predict(tdpd_mlp *m, int n, const float *X, float *mean, fl
         tdpd_status rc = pred_workspace(m, need);
         if (rc) return rc;
         d = m->pred;
-    } else {
-        MCU(cudaMallocAsync((void **)&d, need * sizeof(float), m->st));
+    } else if (cudaMallocAsync((void **)&d, need * sizeof(float), m->st) != cudaSuccess) {
+        cudaGetLastError();                       // (not the next call's error)
+        return mfail(TDPD_ENOMEM, "tdpd_mlp_predict: device allocation failed");
     }
     float *dmean = d + in, *drel = dmean + N * OUT, *dY = drel + N * OUT;
     MCU(cudaMemcpyAsync(d, X, in * sizeof(float), cudaMemcpyHostToDevice, m->st));

@@ -1,12 +1,14 @@
 """The prediction call of the surrogate where its statistics and its workspace can
 go wrong: members or inputs that are not finite, calls of several threads on one
-handle; and the handle after an allocation that failed."""
+handle, sizes around what the workspace keeps; and the handle after an allocation
+that failed."""
 
 import threading
 
 import numpy as np
 import pytest
 
+from oracle import mlp
 from workloads import surrogate as S
 from gpu_common import B
 
@@ -122,3 +124,44 @@ def test_samples_that_do_not_fit_leave_a_usable_handle():
     finally:
         bd.tdpd_mlp_destroy(h)
         bd.tdpd_mlp_destroy(g)
+
+
+def test_prediction_sizes_around_the_workspace():
+    """Two members take 12 floats a point: the largest call that fits what comes with
+    the handle (65,536 floats) and the first that does not, the largest kept (2^22) and
+    the first that allocates for itself; then small calls. Against the oracle (1e-6 of
+    the outputs' magnitude, the rounding of sums of 64 binary32 products)."""
+    bd, members = B(), 2
+    h = _handle(members)
+    P, X0 = S.init_params(11, members), _points(64, 12).astype(np.float64)
+    st = mlp.Standardizer(X0, np.stack([2 + X0[:, 0] * X0[:, 1], 3 + X0[:, 3]], 1).astype(np.float32).astype(np.float64))
+    try:
+        for n in (5461, 5462, 349525, 349526, 31, 5463):
+            X = _points(n, n)
+            mean, spread, each, want = _finite_predictions(h, X, members)
+            at = np.unique(np.r_[0:min(n, 500), max(0, n - 500):n])
+            Xn = st.x(X[at].astype(np.float64)).astype(np.float32).astype(np.float64)
+            for k in range(members):
+                y = st.y_inv(mlp.forward(P[k], Xn)[0])
+                assert np.abs(each[k][at] - y).max() < 1e-6 * np.abs(y).max(), (n, k)
+            assert np.abs(mean - each.astype(np.float64).mean(0)).max() < 1e-6 * np.abs(mean).max(), n
+            assert np.abs(spread - want).max() < 1e-6, n
+    finally:
+        bd.tdpd_mlp_destroy(h)
+
+
+def test_a_call_that_does_not_fit_the_device():
+    """Two thousand million points with 64 members need 1.1 TB: refused before the
+    points are read, and the next call is as before."""
+    bd, members = B(), 64
+    h = _handle(members)
+    X = _points(50, 15)
+    mean = np.zeros((50, 2), np.float32)
+    try:
+        before = bd.tdpd_mlp_predict(h, X, members)
+        rc = bd.lib.tdpd_mlp_predict(h, 2_000_000_000, bd._ptr(X), bd._ptr(mean), None, None)
+        assert bd.STATUS[rc] == 'ENOMEM'
+        for a, b in zip(before, bd.tdpd_mlp_predict(h, X, members)):
+            assert np.array_equal(a, b)
+    finally:
+        bd.tdpd_mlp_destroy(h)
