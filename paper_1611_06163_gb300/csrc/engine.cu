@@ -1715,8 +1715,8 @@ tdpd_status tdpd_add_rbc(tdpd_sys *s, int nv, const float *pos, const float *vel
     if (!s) return fail(nullptr, TDPD_EINVAL, "null handle");
     if (s->committed || s->reps.size() != 1) return fail(s, TDPD_ESTATE, "membranes are fixed after commit or batching");
     HostRep &R = s->reps[0];
-    if (nv < 4 || nv > 1024 || !pos || !vel || !tri || ntri != 2 * nv - 4)
-        return fail(s, TDPD_EINVAL, "membrane needs 4..1024 vertices and 2*nv-4 triangles");
+    if (nv < 4 || nv > MESH_MAX_NV || !pos || !vel || !tri || ntri != 2 * nv - 4)
+        return fail(s, TDPD_EINVAL, "membrane needs 4..%d vertices and 2*nv-4 triangles", MESH_MAX_NV);
     if (type < 0 || type >= R.cfg.n_types) return fail(s, TDPD_EINVAL, "membrane type out of range");
     if ((long)R.type.size() + nv > TDPD_MAX_IDS) return fail(s, TDPD_EOVERFLOW, "more than %d particles", TDPD_MAX_IDS);
     for (int i = 0; i < 3 * nv; ++i) {

@@ -52,10 +52,15 @@ constexpr int REF_THREADS = 256;
 // four vertices (three planes of 4 x the share), of the triangles their area and
 // volume.
 __host__ __device__ constexpr int share_of(int n, int C) { return (n + C - 1) / C; }
-static size_t membrane_smem(int nv, int C)
+static constexpr size_t membrane_smem(int nv, int C)
 {
     return (size_t)nv * 32 + (size_t)share_of(3 * nv - 6, C) * 48 + (size_t)share_of(2 * nv - 4, C) * 8;
 }
+// The launch limits are those of the largest mesh, not of the handle that launches: a
+// kernel's limit belongs to the process, and a handle with a smaller mesh in another
+// thread would lower it between this one's setting and its launch.
+constexpr size_t MEMBRANE_SMEM_MAX = membrane_smem(MESH_MAX_NV, 1);
+static_assert(MEMBRANE_SMEM_MAX + 1024 <= 227 * 1024, "the largest mesh fits one CTA (with the static arrays)");
 
 // C CTAs (a thread-block cluster; CL false: one CTA) per membrane. Each stages all
 // its vertices, computes a share of the edges and triangles and sums a share of
@@ -372,14 +377,13 @@ void launch_mem_ref(const float *x3, const RbcDev *rbcs, const FanEntry *fan, co
     if (n_rbc <= 0) return;
     constexpr size_t SMEM_MAX = 200 * 1024;
     const size_t staged = sizeof(int) * ((size_t)4 * max_nv + (size_t)max_nv * max_stride);
-    const size_t plain = sizeof(int) * (size_t)max_nv;
+    const size_t plain = sizeof(int) * (size_t)max_nv;       // (at most 4 KB)
     if (staged <= SMEM_MAX) {
+        // (the same limit for every handle, as for k_membrane)
         if (staged > 48 * 1024)
-            cudaFuncSetAttribute(k_mem_ref<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)staged);
+            cudaFuncSetAttribute(k_mem_ref<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_MAX);
         k_mem_ref<true><<<n_rbc, REF_THREADS, staged, st>>>(x3, rbcs, fan, reps, ref_out, max_nv, max_stride);
     } else {
-        if (plain > 48 * 1024)
-            cudaFuncSetAttribute(k_mem_ref<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plain);
         k_mem_ref<false><<<n_rbc, REF_THREADS, plain, st>>>(x3, rbcs, fan, reps, ref_out, max_nv, max_stride);
     }
 }
@@ -393,7 +397,8 @@ void launch_membrane(const MemArgs &a, cudaStream_t st, bool pdl)
     const int C = membrane_ctas(a.n_rbc);
     auto kern = C > 1 ? k_membrane<true> : k_membrane<false>;
     const size_t smem = membrane_smem(a.max_nv, C);
-    if (smem > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (smem > 48 * 1024)
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MEMBRANE_SMEM_MAX);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = a.n_rbc * C;
     cfg.blockDim = MEM_THREADS;

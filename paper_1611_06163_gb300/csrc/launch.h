@@ -105,6 +105,8 @@ struct ListArgs {
     int striped;                 // one list per particle (list_striped.cuh), nlc [n]
 };
 
+constexpr int MESH_MAX_NV = 1024;    // vertices of a membrane
+
 struct MemArgs {
     const float4 *mx, *mv;       // vertex position and v~ by load index
     const RepParams *reps;

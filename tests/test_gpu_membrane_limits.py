@@ -1,0 +1,78 @@
+"""The membrane kernel at the limit of its shared memory (one CTA for a mesh of 1024
+vertices), and handles of different meshes committed by several threads at once."""
+
+import threading
+
+import numpy as np
+import pytest
+
+from gpu_common import B, W, make
+
+pytestmark = pytest.mark.gpu
+
+
+def _cell(nv, seed, L=9.0):
+    d = W.single_rbc(L=L, nv=500, diameter=5.0, seed=seed)
+    rng = np.random.default_rng(seed)
+    verts, tri = W.sphere_mesh(nv, 2.2)
+    d['rbcs'] = [W.place_rbc(verts, tri, (0.3, L - 0.2, 0.5 * L), d['L'], rng)]
+    d = W.perturb(d, seed + 1, dx=0.02 * 2.2 / np.sqrt(nv / 12.0), rbc_scale=1.02)
+    return dict(d, lanes=1, pair_mode=2, skin=0.2)
+
+
+def _run(h, replica):
+    bd = B()
+    return bd.tdpd_read_state(h, replica, 1) + bd.tdpd_read_forces(h, replica, 1) + bd.tdpd_read_rbc(h, replica, 1)
+
+
+def test_one_cta_of_the_largest_mesh():
+    """153 membranes take a CTA each; alone a membrane takes four: the same bits."""
+    bd, replicas = B(), 153
+    ds = [_cell(1024, 950 + k % 3) for k in range(replicas)]
+    hs = [bd.create_from(d) for d in ds]
+    b = bd.tdpd_batch_create(hs)
+    for h in hs:
+        bd.tdpd_destroy(h)
+    bd.tdpd_set_lanes(b, 1)
+    bd.tdpd_set_pair_mode(b, 2)
+    bd.tdpd_set_skin(b, 0.2)
+    try:
+        bd.tdpd_step(b, 3)
+        bd.tdpd_sync(b)
+        for k in (0, 1, 2, replicas - 1):
+            h = make(ds[k])
+            bd.tdpd_step(h, 3)
+            bd.tdpd_sync(h)
+            for x, y in zip(_run(b, k), _run(h, 0)):
+                assert np.array_equal(x, y), k
+            bd.tdpd_destroy(h)
+    finally:
+        bd.tdpd_destroy(b)
+
+
+def test_threads_commit_different_meshes():
+    """Both meshes need more shared memory than a launch has by default."""
+    bd = B()
+    want, done = {}, []
+    ds = {nv: _cell(nv, 960) for nv in (700, 1024)}
+
+    def run(nv):
+        h = make(ds[nv])
+        bd.tdpd_step(h, 2)
+        bd.tdpd_sync(h)
+        out = _run(h, 0)
+        bd.tdpd_destroy(h)
+        return out
+
+    def work(nv):
+        for _ in range(8):
+            done.append(all(np.array_equal(x, y) for x, y in zip(run(nv), want[nv])))
+
+    for nv in ds:
+        want[nv] = run(nv)
+    threads = [threading.Thread(target=work, args=(nv,)) for nv in list(ds) * 2]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert len(done) == 32 and all(done)
