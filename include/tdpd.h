@@ -234,9 +234,11 @@ tdpd_status tdpd_list_shape(tdpd_sys *s, float *skin, int *cells_per_cutoff, flo
  * of one thread-block cluster (8 or 16 CTAs) doing all four, its phases
  * separated by the cluster barrier -- for systems of at most 32,768
  * particles (16,384 where only an 8-CTA cluster fits) and 1,048,576 cells,
- * where the chain's launches cost more than its work. Both give the same sorted order and the same bits. With 0,
- * commit times 16 steps of each (graph replays) where the cluster
- * sort fits, and keeps it unless the chain is more than 3 % faster. Before
+ * where the chain's launches cost more than its work. Both give the same sorted
+ * order and the same bits. With 0, commit times 16 steps of each (graph replays) with
+ * the default list shape, before it times others, and keeps the cluster unless the
+ * chain is more than 3 % faster; where the cluster does not serve the default shape,
+ * the chain is used without timing. Before
  * tdpd_commit; TDPD_EINVAL for another value, TDPD_ESTATE after commit;
  * commit fails with TDPD_EINVAL when 2 is set and the cluster sort does not
  * fit (cell mode: the setting is ignored). */

@@ -74,6 +74,8 @@ struct tdpd_sys {
     int mode_fixed = 0;    // pair mode: 0 chosen at commit, 1 full shell, 2 half shell
     int sort_fixed = 0;    // list-mode sort: 0 chosen at commit, 1 kernel chain, 2 one cluster
     int sort_ctas = 0;     // CTAs of the one-cluster sort in use (0: the kernel chain)
+    int sort_ctas_max = 0; // CTAs it has on this device (0: it cannot run)
+    bool sort_chain = false;   // the chain whatever the shape: pinned, timed faster, or no cluster for the default
     std::vector<float> sort_ms;    // commit's timing of the two sorts (ms per 16 steps: cluster, chain)
     std::vector<float> shape_ms;   // commit's timing of the candidate list shapes (ms per 16 steps)
     int shape_win = -1;            // the shape chosen (-1: not timed)
@@ -1135,8 +1137,16 @@ std::vector<Shape> shape_candidates(const tdpd_sys *s)
     return v;
 }
 
-// Make shape (skin, m) current: replica tables, cell count, lists sized and
-// built for the state the host holds, forces evaluated.
+// CTAs of the one-cluster sort for the current shape; 0: the kernel chain, which was
+// timed faster or pinned, or the cluster does not serve this shape's cells.
+int sort_ctas_now(const tdpd_sys *s)
+{
+    if (!s->use_list || s->sort_chain || s->NC > SORT_SMALL_MAX_NC) return 0;
+    return s->N <= s->sort_ctas_max * SORT_SMALL_THREADS * SORT_SMALL_ITEMS ? s->sort_ctas_max : 0;
+}
+
+// Make shape (skin, m) current: replica tables, cell count, the sort that serves it,
+// lists sized and built for the state the host holds, forces evaluated.
 tdpd_status apply_shape(tdpd_sys *s, const Shape &sh)
 {
     std::vector<RepParams> P;
@@ -1145,6 +1155,7 @@ tdpd_status apply_shape(tdpd_sys *s, const Shape &sh)
     if (rc) return rc;
     if (NC > s->n_tiles * SCAN_TILE) return fail(s, TDPD_ESTATE, "cell arrays too small for a tuned shape");
     s->NC = NC;
+    s->sort_ctas = sort_ctas_now(s);
     if ((rc = upload(s, s->d_reps, P.data(), P.size()))) return rc;
     return reload_state(s);
 }
@@ -1172,25 +1183,22 @@ tdpd_status tune_shape(tdpd_sys *s, const std::vector<Shape> &shapes)
     return TDPD_OK;
 }
 
-// CTAs of the one-cluster sort for the current shape; 0: it does not serve it.
-int sort_ctas_allowed(const tdpd_sys *s)
-{
-    const int ctas = s->NC <= SORT_SMALL_MAX_NC ? sort_small_ctas(s->ns) : 0;
-    return s->N <= ctas * SORT_SMALL_THREADS * SORT_SMALL_ITEMS ? ctas : 0;
-}
-
-// List mode: the sort of a step as one cluster launch or as the kernel chain.
-// Both give the same bits; unless the caller pinned one, time steps with each and
-// keep the cluster unless the chain is more than 3 % faster; then reload the
-// host's state.
+// List mode: the sort of a step as one cluster launch or as the kernel chain. Both
+// give the same bits; unless the caller pinned one, time steps of the default shape
+// with each and keep the cluster unless the chain is more than 3 % faster; then reload
+// the host's state. A default shape with too many cells for the cluster takes the
+// chain, and so do the other shapes, although those of a wider skin may fit: near the
+// limit the scan by one cluster is far slower (2,916 particles in 1.03 M cells: 2.35 ms
+// for 16 steps, the chain 0.36).
 tdpd_status tune_sort(tdpd_sys *s)
 {
-    s->sort_ctas = 0;
+    s->sort_chain = s->sort_fixed == 1;
     s->sort_ms.clear();
-    if (!s->use_list || s->sort_fixed == 1) return TDPD_OK;
-    const int ctas = sort_ctas_allowed(s);
-    if (s->sort_fixed == 2) s->sort_ctas = ctas;
-    if (s->sort_fixed == 2 || !ctas) return TDPD_OK;
+    s->sort_ctas = sort_ctas_now(s);
+    if (!s->use_list || s->sort_fixed) return TDPD_OK;
+    s->sort_chain = !s->sort_ctas;
+    if (s->sort_chain) return TDPD_OK;
+    const int ctas = s->sort_ctas;
     float t[2] = {1e30f, 1e30f};
     tdpd_status rc;
     for (int k = 0; k < 2; ++k) {
@@ -1198,22 +1206,11 @@ tdpd_status tune_sort(tdpd_sys *s)
         if ((k && (rc = init_state(s))) || (rc = time_steps(s, &t[k]))) return rc;
     }
     s->sort_ms.assign(t, t + 2);
-    s->sort_ctas = t[0] <= 1.03f * t[1] ? ctas : 0;
+    s->sort_chain = t[0] > 1.03f * t[1];
+    s->sort_ctas = sort_ctas_now(s);
     s->step = 0;
     if ((rc = init_state(s))) return rc;
     if (s->builds) CU(cudaMemsetAsync(s->builds, 0, sizeof(uint32_t) * s->reps.size(), exec_stream(s)));
-    return TDPD_OK;
-}
-
-// The one-cluster sort against the limits of the shape that was kept.
-tdpd_status check_sort(tdpd_sys *s)
-{
-    const int ctas = s->use_list && s->sort_fixed != 1 ? sort_ctas_allowed(s) : 0;
-    if (s->use_list && s->sort_fixed == 2 && !ctas)
-        return fail(s, TDPD_EINVAL, "the one-cluster sort needs at most %d particles and %d cells (here %d, %d) "
-                    "and a resident cluster of 8 or 16 CTAs", 16 * SORT_SMALL_THREADS * SORT_SMALL_ITEMS,
-                    SORT_SMALL_MAX_NC, s->N, s->NC);
-    if (s->sort_fixed == 2 || !ctas) s->sort_ctas = ctas;
     return TDPD_OK;
 }
 
@@ -1498,11 +1495,15 @@ tdpd_status commit(tdpd_sys *s)
     CU(cudaStreamCreateWithFlags(&s->side, cudaStreamNonBlocking));
     CU(cudaEventCreateWithFlags(&s->fork, cudaEventDisableTiming));
     CU(cudaEventCreateWithFlags(&s->join, cudaEventDisableTiming));
-    // the sort first: lanes and shapes are then timed in steps as they will run
+    // the sort first: shapes and lanes are then timed in steps as they will run
+    s->sort_ctas_max = s->use_list ? sort_small_ctas(ns) : 0;
     if ((rc = tune_sort(s))) return rc;
     if (!shapes.empty() && (rc = tune_shape(s, shapes))) return rc;
     if (s->lanes_fixed == 0 && (rc = autotune(s))) return rc;
-    if ((rc = check_sort(s))) return rc;
+    if (s->use_list && s->sort_fixed == 2 && !s->sort_ctas)
+        return fail(s, TDPD_EINVAL, "the one-cluster sort needs at most %d particles and %d cells (here %d, %d) "
+                    "and a resident cluster of 8 or 16 CTAs", 16 * SORT_SMALL_THREADS * SORT_SMALL_ITEMS,
+                    SORT_SMALL_MAX_NC, s->N, s->NC);
     const int nk = (int)step_kernels(s).size();
     for (int k = 0; k <= nk; ++k) CU(cudaEventCreate(&s->ev[k]));
     s->n_ev = nk + 1;
