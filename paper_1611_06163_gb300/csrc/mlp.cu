@@ -9,6 +9,7 @@
 #include <cuda_bf16.h>
 
 #include <cmath>
+#include <cstddef>
 #include <cstring>
 #include <mutex>
 #include <new>
@@ -46,7 +47,8 @@ constexpr int CH = 32;           // samples per CTA
 constexpr int LDS_ = CH + 4;     // padded row of a feature-major activation (16-byte rows)
 constexpr int LDW = HID + 4;     // padded row of W2
 
-struct NetSmem {
+// (aligned for the 16-byte accesses, and every row of them)
+struct alignas(16) NetSmem {
     float W2[HID][LDW];
     float W1[HID][IN];
     float b1[HID], b2[HID], W3[OUT][HID], b3[OUT], pad[2];
@@ -54,6 +56,10 @@ struct NetSmem {
     float H1[HID][LDS_];
     float Y[TPB / 32][OUT][CH];  // each warp's share of the outputs
 };
+
+static_assert(offsetof(NetSmem, W1) % 16 == 0 && offsetof(NetSmem, X) % 16 == 0 && offsetof(NetSmem, H1) % 16 == 0 &&
+              offsetof(NetSmem, Y) % 16 == 0 && LDW % 4 == 0 && LDS_ % 4 == 0 && CH % 4 == 0 && IN == 4,
+              "16-byte rows");
 
 __device__ __forceinline__ void load_net(NetSmem &S, const float *__restrict__ p)
 {
@@ -238,6 +244,7 @@ struct TrainSmem {
     NetSmem N;
     float D2[HID][LDS_];
 };
+static_assert(alignof(TrainSmem) >= 16 && offsetof(TrainSmem, D2) % 16 == 0, "16-byte rows");
 
 // PARTS: the launch takes every PARTS-th chunk, from `first` on, and (first > 0) adds
 // its sums to the row of the chunk before, so that a row of part holds PARTS chunks.
