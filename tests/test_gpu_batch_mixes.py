@@ -46,8 +46,8 @@ def _results(h, ns, replicas):
 
 @pytest.mark.parametrize('mix', [(PLAIN, TYPES), (PLAIN, FLUX), (TYPES, FLUX_TYPES), (FLUX, TYPES), (PLAIN, SOFT)])
 @pytest.mark.parametrize('ns, lanes, mode', [(1, 1, 1), (1, 4, 2), (1, 32, 1), (2, 4, 1), (2, 1, 2), (2, 32, 2),
-                                             (3, 4, 1), (3, 1, 2), (10, 1, 1), (10, 8, 1), (10, 8, 2), (16, 2, 1),
-                                             (1, 2, 0), (2, 2, 0), (3, 8, 0)])
+                                             (3, 4, 1), (3, 1, 2), (5, 4, 1), (8, 8, 2), (10, 1, 1), (10, 8, 1),
+                                             (10, 8, 2), (16, 2, 1), (1, 2, 0), (2, 2, 0), (3, 8, 0)])
 def test_batch_equals_alone_in_mixed_batches(mix, ns, lanes, mode):
     """mode 0: cell mode (skin 0)."""
     bd = B()
@@ -73,6 +73,14 @@ def test_batch_equals_alone_in_mixed_batches(mix, ns, lanes, mode):
                 assert np.array_equal(x, y), k
     finally:
         bd.tdpd_destroy(b)
+
+
+@pytest.mark.parametrize('ns, types, lanes, mode', [(3, 2, 8, 1), (3, 1, 2, 2), (6, 1, 1, 1), (7, 2, 16, 2),
+                                                    (8, 1, 4, 1), (8, 3, 32, 2), (9, 1, 4, 1), (9, 2, 1, 2)])
+def test_forms_by_species_count_match_oracle(ns, types, lanes, mode):
+    d = dict(_box(ns, 70 + ns + lanes, 6.0, types=types), lanes=lanes, pair_mode=mode)
+    F, Q, Fo, Qo = forces_vs_oracle(d)
+    check_step(F, Q, Fo, Qo, (ns, types, lanes, mode))
 
 
 @pytest.mark.parametrize('ns, types, lanes, mode', [(1, 1, 1, 1), (1, 3, 4, 2), (1, 2, 32, 1), (2, 2, 2, 2),
