@@ -44,7 +44,6 @@ __device__ __forceinline__ float3 rel_pos(const RepParams &P, float4 x, float4 r
                        min_image(x.z - ref.z, P.L[2], P.periodic[2]));
 }
 
-constexpr int MEM_THREADS = 512;
 constexpr int REF_THREADS = 256;
 
 // Dynamic shared memory of one of the C CTAs of a membrane: every vertex's
@@ -67,21 +66,24 @@ static_assert(MEMBRANE_SMEM_MAX + 1024 <= 227 * 1024, "the largest mesh fits one
 // the vertices, reading the other shares through distributed shared memory. Every
 // sum has an order of its own, whatever C is (a triangle's terms are added by
 // thread t mod 512, a vertex's fan by eight lanes), so a membrane gives the same
-// bits alone and in a batch.
+// bits alone and in a batch. T threads: 512, or 128 for meshes of at most 128
+// triangles, whose sums have the same order with either (the other threads of 512 add
+// zeros).
 //
 // Bound by the arithmetic, above all the five TEA draws and ten normals of a
 // bond's random force (about 650 of 900 instructions per edge). Computed from each
 // of its ends, with the dihedral from each of its four vertices (eight lanes per
 // vertex over its fan), this took 47 us on the 229 cells of 128 replicas after a
 // K-Gather of 8 us; every edge once: 38 us in one launch. A single cell is a chain of
-// latencies: 22 us in one CTA, 12.4 in four (12.0 in the two kernels before).
-template <bool CL>
-__global__ void __launch_bounds__(MEM_THREADS, 2) k_membrane(MemArgs A)
+// latencies, split over the CTAs (membrane_ctas).
+constexpr int MEM_THREADS = 512, MEM_THREADS_SMALL = 128;
+template <bool CL, int T>
+__global__ void __launch_bounds__(T, 1024 / T) k_membrane(MemArgs A)
 {
     namespace cg = cooperative_groups;
     pdl_enter();
     extern __shared__ float4 mem_sm[];
-    __shared__ FF sh[MEM_THREADS / 32][5];
+    __shared__ FF sh[T / 32][5];
     __shared__ float2 cgv_sh;
     cg::cluster_group cl = cg::this_cluster();
     const int C = CL ? (int)cl.num_blocks() : 1, rank = CL ? (int)cl.block_rank() : 0;
@@ -104,7 +106,7 @@ __global__ void __launch_bounds__(MEM_THREADS, 2) k_membrane(MemArgs A)
     FF v[5];
 #pragma unroll
     for (int k = 0; k < 5; ++k) v[k] = FF{0.0f, 0.0f};
-    for (int k = tid; k < R.nv; k += MEM_THREADS) {
+    for (int k = tid; k < R.nv; k += T) {
         const float3 x = rel_pos(P, A.mx[R.gbase + k], ref);
         xs[k] = make_float4(x.x, x.y, x.z, 0.0f);
         vs[k] = A.mv[R.gbase + k];
@@ -113,7 +115,7 @@ __global__ void __launch_bounds__(MEM_THREADS, 2) k_membrane(MemArgs A)
         v[4] = ff_add(v[4], x.z);
     }
     __syncthreads();
-    for (int t = tp; t < t1; t += MEM_THREADS) {
+    for (int t = tp; t < t1; t += T) {
         if (t != tp) tv = make_int3(tri[3 * t], tri[3 * t + 1], tri[3 * t + 2]);
         const float3 x0 = f3(xs[tv.x]), x1 = f3(xs[tv.y]), x2 = f3(xs[tv.z]);
         const float3 n = cross(sub(x1, x0), sub(x2, x0));
@@ -123,7 +125,7 @@ __global__ void __launch_bounds__(MEM_THREADS, 2) k_membrane(MemArgs A)
     {
         const uint32_t step = A.mem_ctr[A.q] + P.step0;
         const int id0 = R.gbase - P.pbase;
-        for (int e = ep; e < e1; e += MEM_THREADS) {
+        for (int e = ep; e < e1; e += T) {
             if (e != ep) E = A.edge[R.edge_off + e];
             const float2 bp = A.bond[R.bond_off + e];        // (l_m, k_p)
             const float3 xa = f3(xs[E.x]), xb = f3(xs[E.y]), xc = f3(xs[E.z]), xd = f3(xs[E.w]);
@@ -187,7 +189,7 @@ __global__ void __launch_bounds__(MEM_THREADS, 2) k_membrane(MemArgs A)
 
     // the totals, by every CTA of the membrane
     const int lane = tid & 31, w = tid >> 5;
-    for (int t = tid; t < R.ntri; t += MEM_THREADS) {
+    for (int t = tid; t < R.ntri; t += T) {
         float2 av;
         if (CL) {
             const int r = t / ts;
@@ -206,7 +208,7 @@ __global__ void __launch_bounds__(MEM_THREADS, 2) k_membrane(MemArgs A)
         for (int k = 0; k < 5; ++k) sh[w][k] = v[k];
     __syncthreads();
     if (w == 0) {
-        constexpr int NW = MEM_THREADS / 32;
+        constexpr int NW = T / 32;
 #pragma unroll
         for (int k = 0; k < 5; ++k) v[k] = lane < NW ? sh[lane][k] : FF{0.0f, 0.0f};
 #pragma unroll
@@ -250,7 +252,7 @@ __global__ void __launch_bounds__(MEM_THREADS, 2) k_membrane(MemArgs A)
         }
         return make_float3(o[0], o[4 * es], o[8 * es]);
     };
-    for (int k0 = v0; k0 < v1; k0 += MEM_THREADS / 8) {
+    for (int k0 = v0; k0 < v1; k0 += T / 8) {
         const int k = k0 + (tid >> 3);
         float3 f = make_float3(0.f, 0.f, 0.f);
         if (k < v1) {
@@ -388,20 +390,45 @@ void launch_mem_ref(const float *x3, const RbcDev *rbcs, const FanEntry *fan, co
     }
 }
 
-// CTAs per membrane: the most (of 1, 2, 4) that leave one to two CTAs per SM
-static int membrane_ctas(int n_rbc) { return n_rbc <= 76 ? 4 : n_rbc <= 152 ? 2 : 1; }
+// CTAs per membrane: the most that leave one CTA per SM (clusters of eight and four
+// fill a little less than 152 SMs), since a second wave, or a second CTA on every SM,
+// costs more than the split gains; eight only for meshes of more than 512 vertices
+// (beside the half shell's pair walk eight CTAs of one mesh of 500 vertices delay it by
+// as much as they finish earlier: 32.1 us per step with four, 32.5); beyond 152
+// membranes one, which then share the SMs two by two, and two for meshes so large that
+// one CTA fills an SM's shared memory. Measured (launch by launch, us, with 1, 2, 4 and 8 CTAs, in brackets the two kernels
+// with a lane per fan entry that this one replaced): 10 meshes of 500 vertices 26.6,
+// 20.8, 16.4, 14.3 (22); 36 of 26.6, 20.7, 16.7, 18.4 (24); 76 of 26.6, 20.4, 28.7,
+// 36.9 (32); 152 of 26.6, 28.7, 43, 60 (45); 153 of 37, 39, 43, 60 (47); 300 of 41, 52,
+// 72 (76). 10 of 1000 vertices 40.5, 30.7, 22.5, 18.4 (22); 153 of 82, 64, 66, 80 (76);
+// 300 of 84, 82, 109 (129).
+constexpr size_t SMEM_PER_SM = 228 * 1024;
+static int membrane_ctas(int n_rbc, int max_nv)
+{
+    if (n_rbc <= 152) return n_rbc <= 16 && max_nv > 512 ? 8 : n_rbc <= 36 ? 4 : n_rbc <= 76 ? 2 : 1;
+    return membrane_smem(max_nv, 1) + 2048 > SMEM_PER_SM / 2 ? 2 : 1;
+}
+
+// Many small meshes: with 128 threads eight membranes share an SM (3,000 meshes of 12
+// vertices 29 us, with 512 threads 78, the kernels before 71; 1,000 of 42 vertices 19,
+// 35, 47).
+static int membrane_threads(int ctas, int max_nv)
+{
+    return ctas == 1 && 2 * max_nv - 4 <= MEM_THREADS_SMALL ? MEM_THREADS_SMALL : MEM_THREADS;
+}
 
 void launch_membrane(const MemArgs &a, cudaStream_t st, bool pdl)
 {
     if (a.n_rbc <= 0) return;
-    const int C = membrane_ctas(a.n_rbc);
-    auto kern = C > 1 ? k_membrane<true> : k_membrane<false>;
+    const int C = membrane_ctas(a.n_rbc, a.max_nv), T = membrane_threads(C, a.max_nv);
+    auto kern = C > 1 ? k_membrane<true, MEM_THREADS>
+                : T == MEM_THREADS ? k_membrane<false, MEM_THREADS> : k_membrane<false, MEM_THREADS_SMALL>;
     const size_t smem = membrane_smem(a.max_nv, C);
     if (smem > 48 * 1024)
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MEMBRANE_SMEM_MAX);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = a.n_rbc * C;
-    cfg.blockDim = MEM_THREADS;
+    cfg.blockDim = T;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cudaLaunchAttribute at[2];

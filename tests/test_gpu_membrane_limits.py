@@ -1,5 +1,6 @@
-"""The membrane kernel at the limit of its shared memory (one CTA for a mesh of 1024
-vertices), and handles of different meshes committed by several threads at once."""
+"""The membrane kernel's splits over CTAs and threads, up to the limit of its shared
+memory (one CTA for a mesh of 1024 vertices), and handles of different meshes committed
+by several threads at once."""
 
 import threading
 
@@ -25,10 +26,14 @@ def _run(h, replica):
     return bd.tdpd_read_state(h, replica, 1) + bd.tdpd_read_forces(h, replica, 1) + bd.tdpd_read_rbc(h, replica, 1)
 
 
-def test_one_cta_of_the_largest_mesh():
-    """153 membranes take a CTA each; alone a membrane takes four: the same bits."""
-    bd, replicas = B(), 153
-    ds = [_cell(1024, 950 + k % 3) for k in range(replicas)]
+@pytest.mark.parametrize('sizes, replicas', [((1024,), 100), ((1024, 600), 153), ((4, 66, 12), 153), ((4, 67, 12), 153),
+                                             ((500, 63), 17), ((4, 1024), 37), ((500, 162), 77)])
+def test_same_bits_for_every_split(sizes, replicas):
+    """Alone a membrane takes four CTAs of 512 threads, eight beyond 512 vertices; 17
+    take four each, 37 two, 77 and 100 one, 153 two of the largest meshes, one of the
+    smaller, and of the smallest one with 128 threads."""
+    bd = B()
+    ds = [_cell(sizes[k % len(sizes)], 950 + k % 6) for k in range(replicas)]
     hs = [bd.create_from(d) for d in ds]
     b = bd.tdpd_batch_create(hs)
     for h in hs:
