@@ -623,7 +623,7 @@ void enqueue_step(tdpd_sys *s, int p, cudaStream_t st, cudaEvent_t *ev = nullptr
     if (branch) {
         cudaEventRecord(s->fork, st);
         cudaStreamWaitEvent(s->side, s->fork, 0);
-        launch_membrane(mem_args(s, 1 - p, 1), s->side, false);
+        launch_membrane(mem_args(s, 1 - p, 1), s->side, false, s->half);
         cudaEventRecord(s->join, s->side);
     }
     mark();
@@ -671,7 +671,7 @@ void enqueue_step(tdpd_sys *s, int p, cudaStream_t st, cudaEvent_t *ev = nullptr
         mark();
     }
     if (s->n_rbc && ev) {
-        launch_membrane(mem_args(s, 1 - p, 1), st, true);
+        launch_membrane(mem_args(s, 1 - p, 1), st, true, s->half);
         mark();
     }
     const PairArgs pa = pair_args(s, nxt, 1, s->tile_sum[1 - p], s->disp[1 - p],
@@ -781,7 +781,7 @@ void enqueue_init(tdpd_sys *s, cudaStream_t st, bool branch)
     if (branch) {
         cudaEventRecord(s->fork, st);
         cudaStreamWaitEvent(s->side, s->fork, 0);
-        launch_membrane(mem_args(s, 1, 0), s->side, false);
+        launch_membrane(mem_args(s, 1, 0), s->side, false, s->half);
         cudaEventRecord(s->join, s->side);
     }
     launch_bin_init(s->buf[0], s->d_reps, N, s->count, s->tile_sum[0], s->cellrank, st);
@@ -797,7 +797,7 @@ void enqueue_init(tdpd_sys *s, cudaStream_t st, bool branch)
         launch_rank_gather(s->buf[0], s->buf[1], s->d_reps, s->keys, s->cellrank, s->cell_start, s->inv, N, ns, 0,
                            st, nullptr, 0, nullptr, 0, quarantine(s));
     }
-    if (s->n_rbc && !branch) launch_membrane(mem_args(s, 1, 0), st, true);
+    if (s->n_rbc && !branch) launch_membrane(mem_args(s, 1, 0), st, true, s->half);
     const PairArgs pa = pair_args(s, s->buf[1], 0, s->tile_sum[1], s->disp[1],
                                   s->use_list && pair_builds_lists(s) ? s->rb_all : nullptr);
     if (branch && !s->half) cudaStreamWaitEvent(st, s->join, 0);

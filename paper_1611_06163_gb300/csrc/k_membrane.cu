@@ -61,14 +61,57 @@ static constexpr size_t membrane_smem(int nv, int C)
 constexpr size_t MEMBRANE_SMEM_MAX = membrane_smem(MESH_MAX_NV, 1);
 static_assert(MEMBRANE_SMEM_MAX + 1024 <= 227 * 1024, "the largest mesh fits one CTA (with the static arrays)");
 
+// The sums of K terms over n items, as SUM_THREADS threads would add them (item i by
+// thread i mod SUM_THREADS, the threads by a tree): the T threads of the CTA take the
+// parts of H of them side by side, so T does not change a bit. add(v, i): item i's
+// terms. The sums are in lane 0 of warp 0. Every thread of the CTA calls it.
+constexpr int SUM_THREADS = 512;
+template <int T, int K, class Add>
+__device__ __forceinline__ void totals(FF (&sum)[K], FF (*sh)[K], int n, Add &&add)
+{
+    constexpr int H = SUM_THREADS / T, NW = SUM_THREADS / 32;
+    static_assert(SUM_THREADS % T == 0 && T % 32 == 0, "whole parts of whole warps");
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    FF v[H][K];
+#pragma unroll
+    for (int h = 0; h < H; ++h)
+#pragma unroll
+        for (int k = 0; k < K; ++k) v[h][k] = FF{0.0f, 0.0f};
+    for (int i = threadIdx.x; i < n; i += SUM_THREADS)
+#pragma unroll
+        for (int h = 0; h < H; ++h)
+            if (i + h * T < n) add(v[h], i + h * T);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int h = 0; h < H; ++h)
+#pragma unroll
+            for (int k = 0; k < K; ++k) v[h][k] = ff_add(v[h][k], ff_shfl_down(v[h][k], o));
+    if (lane == 0)
+#pragma unroll
+        for (int h = 0; h < H; ++h)
+#pragma unroll
+            for (int k = 0; k < K; ++k) sh[h * (T / 32) + w][k] = v[h][k];
+    __syncthreads();
+    if (w != 0) return;
+#pragma unroll
+    for (int k = 0; k < K; ++k) sum[k] = lane < NW ? sh[lane][k] : FF{0.0f, 0.0f};
+#pragma unroll
+    for (int o = NW / 2; o > 0; o >>= 1)
+#pragma unroll
+        for (int k = 0; k < K; ++k) sum[k] = ff_add(sum[k], ff_shfl_down(sum[k], o));
+}
+
 // C CTAs (a thread-block cluster; CL false: one CTA) per membrane. Each stages all
 // its vertices, computes a share of the edges and triangles and sums a share of
 // the vertices, reading the other shares through distributed shared memory. Every
-// sum has an order of its own, whatever C is (a triangle's terms are added by
-// thread t mod 512, a vertex's fan by eight lanes), so a membrane gives the same
-// bits alone and in a batch. T threads: 512, or 128 for meshes of at most 128
-// triangles, whose sums have the same order with either (the other threads of 512 add
-// zeros).
+// sum has an order of its own, whatever C and T (the threads) are: the terms of a
+// total are added as by SUM_THREADS threads, T of them at a time, a vertex's fan by
+// eight lanes. So a membrane gives the same bits alone and in a batch.
+//
+// Every CTA adds the areas and volumes itself; a lagged membrane's are for the next
+// step only, and one CTA of a cluster adds them while the others, which need not wait,
+// sum the vertices.
 //
 // Bound by the arithmetic, above all the five TEA draws and ten normals of a
 // bond's random force (about 650 of 900 instructions per edge). Computed from each
@@ -76,14 +119,13 @@ static_assert(MEMBRANE_SMEM_MAX + 1024 <= 227 * 1024, "the largest mesh fits one
 // vertex over its fan), this took 47 us on the 229 cells of 128 replicas after a
 // K-Gather of 8 us; every edge once: 38 us in one launch. A single cell is a chain of
 // latencies, split over the CTAs (membrane_ctas).
-constexpr int MEM_THREADS = 512, MEM_THREADS_SMALL = 128;
 template <bool CL, int T>
 __global__ void __launch_bounds__(T, 1024 / T) k_membrane(MemArgs A)
 {
     namespace cg = cooperative_groups;
     pdl_enter();
     extern __shared__ float4 mem_sm[];
-    __shared__ FF sh[T / 32][5];
+    __shared__ FF sh_av[SUM_THREADS / 32][2], sh_c[SUM_THREADS / 32][3];
     __shared__ float2 cgv_sh;
     cg::cluster_group cl = cg::this_cluster();
     const int C = CL ? (int)cl.num_blocks() : 1, rank = CL ? (int)cl.block_rank() : 0;
@@ -103,16 +145,10 @@ __global__ void __launch_bounds__(T, 1024 / T) k_membrane(MemArgs A)
     const int tp = t0 + tid, ep = e0 + tid;
     int3 tv = tp < t1 ? make_int3(tri[3 * tp], tri[3 * tp + 1], tri[3 * tp + 2]) : make_int3(0, 0, 0);
     int4 E = ep < e1 ? A.edge[R.edge_off + ep] : make_int4(0, 0, 0, 0);
-    FF v[5];
-#pragma unroll
-    for (int k = 0; k < 5; ++k) v[k] = FF{0.0f, 0.0f};
     for (int k = tid; k < R.nv; k += T) {
         const float3 x = rel_pos(P, A.mx[R.gbase + k], ref);
         xs[k] = make_float4(x.x, x.y, x.z, 0.0f);
         vs[k] = A.mv[R.gbase + k];
-        v[2] = ff_add(v[2], x.x);
-        v[3] = ff_add(v[3], x.y);
-        v[4] = ff_add(v[4], x.z);
     }
     __syncthreads();
     for (int t = tp; t < t1; t += T) {
@@ -187,60 +223,40 @@ __global__ void __launch_bounds__(T, 1024 / T) k_membrane(MemArgs A)
     if (CL) cl.sync();
     else __syncthreads();
 
-    // the totals, by every CTA of the membrane
-    const int lane = tid & 31, w = tid >> 5;
-    for (int t = tid; t < R.ntri; t += T) {
-        float2 av;
-        if (CL) {
-            const int r = t / ts;
-            av = cl.map_shared_rank(tri_av, r)[t - r * ts];
-        } else {
-            av = tri_av[t];
-        }
-        v[0] = ff_add(v[0], av.x);
-        v[1] = ff_add(v[1], av.y);
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-        for (int k = 0; k < 5; ++k) v[k] = ff_add(v[k], ff_shfl_down(v[k], o));
-    if (lane == 0)
-        for (int k = 0; k < 5; ++k) sh[w][k] = v[k];
-    __syncthreads();
-    if (w == 0) {
-        constexpr int NW = T / 32;
-#pragma unroll
-        for (int k = 0; k < 5; ++k) v[k] = lane < NW ? sh[lane][k] : FF{0.0f, 0.0f};
-#pragma unroll
-        for (int o = NW / 2; o > 0; o >>= 1)
-#pragma unroll
-            for (int k = 0; k < 5; ++k) v[k] = ff_add(v[k], ff_shfl_down(v[k], o));
-        if (lane == 0) {
+    // the area and the volume: by every CTA of the membrane, or by the last one of a
+    // lagged membrane's, whose forces use the previous step's coefficients
+    const bool lagged = P.m_lagged && A.cgv_lag, last = rank == C - 1;
+    if (!lagged || last) {
+        FF v[2];
+        totals<T, 2>(v, sh_av, R.ntri, [&](FF (&u)[2], int t) {
+            float2 av;
+            if (CL) {
+                const int r = t / ts;
+                av = cl.map_shared_rank(tri_av, r)[t - r * ts];
+            } else {
+                av = tri_av[t];
+            }
+            u[0] = ff_add(u[0], av.x);
+            u[1] = ff_add(u[1], av.y);
+        });
+        if (tid == 0) {
             const double Ab = ff_value(v[0]), Vb = ff_value(v[1]);
             // constraint coefficients of Eq. 14-15, once per membrane in binary64
-            // (divisions by A0, V0 and nv were done once on the host)
-            const float2 cgv = make_float2((float)((Ab - R.A0) * R.kgA0), (float)((Vb - R.V0) * R.kvV0));
-            cgv_sh = P.m_lagged && A.cgv_lag ? A.cgv_lag[b] : cgv;
-            if (rank == 0) {
+            // (divisions by A0 and V0 were done once on the host)
+            cgv_sh = make_float2((float)((Ab - R.A0) * R.kgA0), (float)((Vb - R.V0) * R.kvV0));
+            if (last) {
                 A.av_out[b] = make_double2(Ab, Vb);
-                A.cgv_out[b] = cgv;
-                const double inv = R.inv_nv;
-                float c3[3] = {(float)(ref.x + ff_value(v[2]) * inv), (float)(ref.y + ff_value(v[3]) * inv),
-                               (float)(ref.z + ff_value(v[4]) * inv)};
-                for (int c = 0; c < 3; ++c)
-                    if (P.periodic[c]) {
-                        if (c3[c] < 0.0f) c3[c] += P.L[c];
-                        else if (c3[c] >= P.L[c]) c3[c] -= P.L[c];
-                    }
-                A.ref_out[b] = make_float4(c3[0], c3[1], c3[2], 0.0f);
+                A.cgv_out[b] = cgv_sh;
             }
         }
+        __syncthreads();
     }
-    __syncthreads();
 
     // a share of the vertices, eight lanes each over the fan
-    const float c_area = cgv_sh.x, c_vol = cgv_sh.y;
-    const int vsh = share_of(R.nv, C), v0 = rank * vsh, v1 = min(v0 + vsh, R.nv);
+    const float2 coef = lagged ? A.cgv_lag[b] : cgv_sh;
+    const float c_area = coef.x, c_vol = coef.y;
+    const int parts = lagged && C > 1 ? C - 1 : C;
+    const int vsh = share_of(R.nv, parts), v0 = rank * vsh, v1 = rank < parts ? min(v0 + vsh, R.nv) : v0;
     auto edge_force = [&](int code) {
         const int role = code >> 29, e = code & ((1 << 29) - 1);
         const float *o;
@@ -281,6 +297,27 @@ __global__ void __launch_bounds__(T, 1024 / T) k_membrane(MemArgs A)
             f.z += __shfl_xor_sync(0xffffffffu, f.z, o);
         }
         if (k < v1 && (tid & 7) == 0) A.fext[R.gbase + k] = make_float4(f.x, f.y, f.z, 0.0f);
+    }
+    if (last) {
+        // the vertex centroid: the next reference point
+        FF v[3];
+        totals<T, 3>(v, sh_c, R.nv, [&](FF (&u)[3], int k) {
+            const float4 x = xs[k];
+            u[0] = ff_add(u[0], x.x);
+            u[1] = ff_add(u[1], x.y);
+            u[2] = ff_add(u[2], x.z);
+        });
+        if (tid == 0) {
+            const double inv = R.inv_nv;
+            float c3[3] = {(float)(ref.x + ff_value(v[0]) * inv), (float)(ref.y + ff_value(v[1]) * inv),
+                           (float)(ref.z + ff_value(v[2]) * inv)};
+            for (int c = 0; c < 3; ++c)
+                if (P.periodic[c]) {
+                    if (c3[c] < 0.0f) c3[c] += P.L[c];
+                    else if (c3[c] >= P.L[c]) c3[c] -= P.L[c];
+                }
+            A.ref_out[b] = make_float4(c3[0], c3[1], c3[2], 0.0f);
+        }
     }
     if (CL) cl.sync();                 // the shares stay until every CTA has read them
 }
@@ -390,45 +427,44 @@ void launch_mem_ref(const float *x3, const RbcDev *rbcs, const FanEntry *fan, co
     }
 }
 
-// CTAs per membrane: the most that leave one CTA per SM (clusters of eight and four
-// fill a little less than 152 SMs), since a second wave, or a second CTA on every SM,
-// costs more than the split gains; eight only for meshes of more than 512 vertices
-// (beside the half shell's pair walk eight CTAs of one mesh of 500 vertices delay it by
-// as much as they finish earlier: 32.1 us per step with four, 32.5); beyond 152
-// membranes one, which then share the SMs two by two, and two for meshes so large that
-// one CTA fills an SM's shared memory. Measured (launch by launch, us, with 1, 2, 4 and 8 CTAs, in brackets the two kernels
-// with a lane per fan entry that this one replaced): 10 meshes of 500 vertices 26.6,
-// 20.8, 16.4, 14.3 (22); 36 of 26.6, 20.7, 16.7, 18.4 (24); 76 of 26.6, 20.4, 28.7,
-// 36.9 (32); 152 of 26.6, 28.7, 43, 60 (45); 153 of 37, 39, 43, 60 (47); 300 of 41, 52,
-// 72 (76). 10 of 1000 vertices 40.5, 30.7, 22.5, 18.4 (22); 153 of 82, 64, 66, 80 (76);
-// 300 of 84, 82, 109 (129).
+// CTAs and threads per membrane: the most CTAs that leave one per SM (clusters of eight
+// and four fill a little less than 152 SMs), since a second wave, or a second CTA on
+// every SM, costs more than the split gains; beyond 152 membranes one, which then share
+// the SMs two by two, and two for meshes so large that one CTA fills an SM's shared
+// memory. Measured, launch by launch, us, with 1, 2, 4 and 8 CTAs of 512 threads (in
+// brackets the two kernels with a lane per fan entry that this one replaced): 10 meshes
+// of 500 vertices 26.6, 20.8, 16.4, 14.3 (22); 36 of 26.6, 20.7, 16.7, 18.4 (24); 76 of
+// 26.6, 20.4, 28.7, 36.9 (32); 152 of 26.6, 28.7, 43, 60 (45); 153 of 37, 39, 43, 60
+// (47); 300 of 41, 52, 72 (76). 10 of 1000 vertices 40.5, 30.7, 22.5, 18.4 (22); 153 of
+// 82, 64, 66, 80 (76); 300 of 84, 82, 109 (129).
+// Beside the half shell's walk a few membranes take smaller CTAs, which disturb it less
+// (a cell in 20^3, eight lanes, us per step: 31.3 with 8 x 256 threads, 32.4 with
+// 8 x 512, 31.9 with 4 x 512; the full shell, which waits for them, 36.4, 35.6 and 36.9).
+// Many small meshes: with 128 threads eight of them share an SM (3,000 meshes of 12
+// vertices 29 us, with 512 threads 78, the kernels before 71; 1,000 of 42 19, 35, 47).
+struct MembraneSplit { int ctas, threads; };
 constexpr size_t SMEM_PER_SM = 228 * 1024;
-static int membrane_ctas(int n_rbc, int max_nv)
+static MembraneSplit membrane_split(int n_rbc, int max_nv, bool beside_walk)
 {
-    if (n_rbc <= 152) return n_rbc <= 16 && max_nv > 512 ? 8 : n_rbc <= 36 ? 4 : n_rbc <= 76 ? 2 : 1;
-    return membrane_smem(max_nv, 1) + 2048 > SMEM_PER_SM / 2 ? 2 : 1;
+    if (n_rbc <= 16) return {8, beside_walk && max_nv <= 512 ? 256 : 512};
+    if (n_rbc <= 152) return {n_rbc <= 36 ? 4 : n_rbc <= 76 ? 2 : 1, 512};
+    if (membrane_smem(max_nv, 1) + 2048 > SMEM_PER_SM / 2) return {2, 512};
+    return {1, max_nv <= 66 ? 128 : 512};
 }
 
-// Many small meshes: with 128 threads eight membranes share an SM (3,000 meshes of 12
-// vertices 29 us, with 512 threads 78, the kernels before 71; 1,000 of 42 vertices 19,
-// 35, 47).
-static int membrane_threads(int ctas, int max_nv)
-{
-    return ctas == 1 && 2 * max_nv - 4 <= MEM_THREADS_SMALL ? MEM_THREADS_SMALL : MEM_THREADS;
-}
-
-void launch_membrane(const MemArgs &a, cudaStream_t st, bool pdl)
+void launch_membrane(const MemArgs &a, cudaStream_t st, bool pdl, bool beside_walk)
 {
     if (a.n_rbc <= 0) return;
-    const int C = membrane_ctas(a.n_rbc, a.max_nv), T = membrane_threads(C, a.max_nv);
-    auto kern = C > 1 ? k_membrane<true, MEM_THREADS>
-                : T == MEM_THREADS ? k_membrane<false, MEM_THREADS> : k_membrane<false, MEM_THREADS_SMALL>;
+    const MembraneSplit split = membrane_split(a.n_rbc, a.max_nv, beside_walk);
+    const int C = split.ctas;
+    auto kern = C == 1 ? (split.threads == 128 ? k_membrane<false, 128> : k_membrane<false, 512>)
+                       : (split.threads == 256 ? k_membrane<true, 256> : k_membrane<true, 512>);
     const size_t smem = membrane_smem(a.max_nv, C);
     if (smem > 48 * 1024)
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MEMBRANE_SMEM_MAX);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = a.n_rbc * C;
-    cfg.blockDim = T;
+    cfg.blockDim = split.threads;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cudaLaunchAttribute at[2];

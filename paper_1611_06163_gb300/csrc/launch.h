@@ -237,8 +237,9 @@ void launch_list_build(const ListArgs &a, cudaStream_t st);
 // largest vertex count and fan stride of the membranes
 void launch_mem_ref(const float *x3, const RbcDev *rbcs, const FanEntry *fan, const RepParams *reps, float4 *ref_out,
                     int n_rbc, int max_nv, int max_stride, cudaStream_t st);
-// pdl: launched as a programmatic dependent of the previous kernel on st
-void launch_membrane(const MemArgs &a, cudaStream_t st, bool pdl);
+// pdl: launched as a programmatic dependent of the previous kernel on st; beside_walk:
+// it runs beside the pair walk (the half shell), which does not wait for it
+void launch_membrane(const MemArgs &a, cudaStream_t st, bool pdl, bool beside_walk);
 // chunks: (replica, first slot, end slot); part: OBS_K doubles per chunk;
 // total: their sums over the chunks in chunk order (binary64); done: a
 // counter at zero, left at zero

@@ -26,20 +26,26 @@ def _run(h, replica):
     return bd.tdpd_read_state(h, replica, 1) + bd.tdpd_read_forces(h, replica, 1) + bd.tdpd_read_rbc(h, replica, 1)
 
 
+@pytest.mark.parametrize('mode', [1, 2])
+@pytest.mark.parametrize('lagged', [0, 1])
 @pytest.mark.parametrize('sizes, replicas', [((1024,), 100), ((1024, 600), 153), ((4, 66, 12), 153), ((4, 67, 12), 153),
-                                             ((500, 63), 17), ((4, 1024), 37), ((500, 162), 77)])
-def test_same_bits_for_every_split(sizes, replicas):
-    """Alone a membrane takes four CTAs of 512 threads, eight beyond 512 vertices; 17
-    take four each, 37 two, 77 and 100 one, 153 two of the largest meshes, one of the
-    smaller, and of the smallest one with 128 threads."""
+                                             ((500, 63), 17), ((4, 1024), 37), ((500, 162), 77), ((513, 4), 16)])
+def test_same_bits_for_every_split(sizes, replicas, lagged, mode):
+    """Up to 16 membranes take eight CTAs of 512 threads each, of 256 beside the half
+    shell's walk for at most 512 vertices; 17 take four, 37 two, 77 and 100 one, 153 two
+    of the largest meshes, one of the smaller, and of the smallest one with 128
+    threads: the same bits alone and in a batch, over steps that pass totals on to the
+    next (a lagged membrane's are added by one CTA of the cluster)."""
     bd = B()
-    ds = [_cell(sizes[k % len(sizes)], 950 + k % 6) for k in range(replicas)]
+    ds = [dict(_cell(sizes[k % len(sizes)], 950 + k % 6), pair_mode=mode) for k in range(replicas)]
+    for d in ds:
+        d['membrane'] = dict(d['membrane'], lagged_av=lagged)
     hs = [bd.create_from(d) for d in ds]
     b = bd.tdpd_batch_create(hs)
     for h in hs:
         bd.tdpd_destroy(h)
     bd.tdpd_set_lanes(b, 1)
-    bd.tdpd_set_pair_mode(b, 2)
+    bd.tdpd_set_pair_mode(b, mode)
     bd.tdpd_set_skin(b, 0.2)
     try:
         bd.tdpd_step(b, 3)
