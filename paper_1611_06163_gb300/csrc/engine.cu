@@ -923,7 +923,7 @@ tdpd_status time_steps(tdpd_sys *s, float *ms)
 // lists, the full shell (every pair from both sides) against the half shell
 // (each pair once, partner shares by fixed-point atomics), unless the mode is
 // pinned. The fastest of five timed launches per candidate; the candidates
-// within 10 % of the best (30 % for the best of a shell) are then timed as whole
+// within 10 % of the best of their shell are then timed as whole
 // steps (time_steps); the first within 3 % of the best of those, half shell before full and fewer lanes
 // before more (they are no slower once the caches are cold, and near-equal
 // times would otherwise flip between runs). The state is then rebuilt with
@@ -986,16 +986,20 @@ tdpd_status autotune(tdpd_sys *s)
     }
     float best = 1e30f;
     for (const auto &x : t) best = std::min(best, x.ms);
-    // the candidates within 10 % of the fastest launch, and the fastest of the other
-    // shell if it is within 30 %, are timed again as whole steps, which is what they will run as: the
-    // launch alone misjudges the half shell's finishing pass and the membrane
-    // forces, which the full shell waits for and the half shell overlaps (a
-    // membrane in 12^3: 30 us a step against 39, pair launches 21 and 20)
+    // the candidates within 10 % of the fastest launch of their shell, unless that is
+    // 30 % above the other shell's, are timed again as whole steps, which is what they
+    // will run as: the launch alone misjudges the half shell's finishing pass and the
+    // membrane forces, which the full shell waits for and the half shell overlaps (a
+    // membrane in 12^3: 30 us a step against 39, pair launches 21 and 20), so the two
+    // shells' launches say little about one another (a cell in 15^3, half shell, 8 and
+    // 16 lanes: launches 23.5 and 23.3 us, steps 24.4 and 29.3; within 10 % of the full
+    // shell's 20.4 the choice fell on either)
     std::vector<Cand> fin;
     for (const auto &x : t) {
-        bool first = true;
-        for (const auto &y : t) first = first && (y.mode != x.mode || x.ms <= y.ms);
-        if (x.ms <= (first ? 1.30f : 1.10f) * best) fin.push_back(x);
+        float shell = 1e30f;
+        for (const auto &y : t)
+            if (y.mode == x.mode) shell = std::min(shell, y.ms);
+        if (shell <= 1.30f * best && x.ms <= 1.10f * shell) fin.push_back(x);
     }
     if (fin.size() > 1) {
         float bstep = 1e30f;
