@@ -923,8 +923,8 @@ tdpd_status time_steps(tdpd_sys *s, float *ms)
 // lists, the full shell (every pair from both sides) against the half shell
 // (each pair once, partner shares by fixed-point atomics), unless the mode is
 // pinned. The fastest of five timed launches per candidate; the candidates
-// within 10 % of the best of their shell are then timed as whole
-// steps (time_steps); the first within 3 % of the best of those, half shell before full and fewer lanes
+// within 10 % of the best (and, of short launches, of their shell's best) are then
+// timed as whole steps (time_steps); the first within 3 % of the best of those, half shell before full and fewer lanes
 // before more (they are no slower once the caches are cold, and near-equal
 // times would otherwise flip between runs). The state is then rebuilt with
 // the winner.
@@ -986,20 +986,22 @@ tdpd_status autotune(tdpd_sys *s)
     }
     float best = 1e30f;
     for (const auto &x : t) best = std::min(best, x.ms);
-    // the candidates within 10 % of the fastest launch of their shell, unless that is
-    // 30 % above the other shell's, are timed again as whole steps, which is what they
+    // the candidates within 10 % of the fastest launch, and the fastest of the other
+    // shell if it is within 30 %, are timed again as whole steps, which is what they
     // will run as: the launch alone misjudges the half shell's finishing pass and the
     // membrane forces, which the full shell waits for and the half shell overlaps (a
-    // membrane in 12^3: 30 us a step against 39, pair launches 21 and 20), so the two
-    // shells' launches say little about one another (a cell in 15^3, half shell, 8 and
-    // 16 lanes: launches 23.5 and 23.3 us, steps 24.4 and 29.3; within 10 % of the full
-    // shell's 20.4 the choice fell on either)
+    // membrane in 12^3: 30 us a step against 39, pair launches 21 and 20). Of launches
+    // as short as these the other shell's within 10 % of its own fastest are timed too
+    // (a cell in 15^3, half shell, 8 and 16 lanes: launches 23.5 and 23.3 us, steps 24.4
+    // and 29.3; the launches alone chose either)
+    constexpr float SHORT_MS = 0.06f;
     std::vector<Cand> fin;
     for (const auto &x : t) {
         float shell = 1e30f;
         for (const auto &y : t)
             if (y.mode == x.mode) shell = std::min(shell, y.ms);
-        if (shell <= 1.30f * best && x.ms <= 1.10f * shell) fin.push_back(x);
+        const bool near = x.ms <= 1.10f * best || x.ms <= (best < SHORT_MS ? 1.10f : 1.0f) * shell;
+        if (near && shell <= 1.30f * best) fin.push_back(x);
     }
     if (fin.size() > 1) {
         float bstep = 1e30f;
