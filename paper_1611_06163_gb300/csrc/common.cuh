@@ -85,19 +85,17 @@ struct RingEntry {
     int nb;       // neighbour vertex nb[l]
     int edge;     // edge index of (v, nb[l])
     int tri;      // triangle index of (v, nb[l], nb[l+1])
-    int across;   // vertex opposite v across the edge (nb[l], nb[l+1])
 };
 
 // The device form of fan entry l of vertex v, at a fixed stride per vertex
-// (entry v * fan_stride + l of its mesh), with the cyclic neighbours nb[l+1]
-// and nb[l-1] included: a lane reaches all its vertex indices with one
-// 32-byte load and no offset table. Entries past the degree have nb = -1.
+// (entry v * fan_stride + l of its mesh), with the next neighbour nb[l+1]
+// included: a lane reaches all its indices with one 32-byte sector and no offset
+// table. Entries past the degree have nb = -1.
 // end, opp: where k_membrane leaves the forces on v of the edges (v, nb[l]) and
 // (nb[l], nb[l+1]): the edge's index, v's place in its table entry << 29.
-struct __align__(16) FanEntry {
-    int nb, edge, tri, across;
-    int nb_next, nb_prev;
-    int end, opp;
+struct __align__(32) FanEntry {
+    int nb, nb_next, end, opp;
+    int tri;
 };
 
 // Programmatic dependent launch: let the next kernel in the stream begin

@@ -243,7 +243,6 @@ tdpd_status build_topo(tdpd_sys *s, int nv, int ntri, const int32_t *tri, Topo &
             E.nb = a;
             E.edge = eid(v, a);
             E.tri = ftri[v][a];
-            E.across = opp[std::make_pair(b, a)];
             T.ring.push_back(E);
             a = b;
         }
@@ -1415,14 +1414,14 @@ tdpd_status commit(tdpd_sys *s)
             for (int v = 0; v < T.nv; ++v) {
                 const int o = T.ring_off[v], deg = T.ring_off[v + 1] - o;
                 for (int l = 0; l < mx; ++l) {
-                    FanEntry F{-1, -1, -1, -1, -1, -1, 0, 0};
+                    FanEntry F{-1, -1, 0, 0, -1};
                     if (l < deg) {
                         const RingEntry &E = T.ring[o + l];
                         // the fan's triangle (v, nb, next) holds nb -> next
                         const int next = T.ring[o + (l + 1) % deg].nb;
                         const int far = T.edge_id.at(std::make_pair(std::min(E.nb, next), std::max(E.nb, next)));
-                        F = FanEntry{E.nb, E.edge, E.tri, E.across, next, T.ring[o + (l + deg - 1) % deg].nb,
-                                     E.edge | (v < E.nb ? 0 : 1) << 29, far | (E.nb < next ? 2 : 3) << 29};
+                        F = FanEntry{E.nb, next, E.edge | (v < E.nb ? 0 : 1) << 29, far | (E.nb < next ? 2 : 3) << 29,
+                                     E.tri};
                     }
                     fan.push_back(F);
                 }
