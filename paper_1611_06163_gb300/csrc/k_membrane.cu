@@ -1,5 +1,5 @@
-// Membrane forces of the triangulated RBC model (Sec. 2.2, Eq. 10-16), one CTA per
-// membrane (k_membrane):
+// Membrane forces of the triangulated RBC model (Sec. 2.2, Eq. 10-16), one CTA or a
+// cluster of CTAs per membrane (k_membrane):
 //   - K-Gather of Sec. 3.3: the triangle areas and signed tetrahedron volumes and
 //     the vertex centroid (the next step's reference point), binary32 terms in
 //     compensated float-float sums, converted to binary64 once, and the
